@@ -418,8 +418,9 @@ __device__ __forceinline__ void bwd_far_pair(const float *__restrict__ tile, con
 // target; past that a pair stays in the FP32 sums).
 constexpr int kBwdCloseList = 64;
 
-// Near and loose tiles on the paired layout, one source at a time (lane x of
-// the accumulators), the self pair excluded by index.  Separations are formed
+// Near and loose tiles on the paired layout: the pair terms of two sources at
+// a time in FP32x2, the sums source by source in order (lane x of the
+// accumulators), the self pair excluded by index.  Separations are formed
 // from both offsets' high and low parts, d = (s - t) + (s_lo - t_lo) (lo: the
 // tile's planes of low parts; tl: the targets'), so they are good to a few
 // units in the last place of d however far the tile centre lies.  A pair
@@ -435,45 +436,61 @@ __device__ __forceinline__ void bwd_near_pair(const float *__restrict__ tile,
 {
     const float hinv3 = hinv * hinv * hinv;
     const float hinv5 = hinv3 * hinv * hinv;
+    const float4 *P0 = reinterpret_cast<const float4 *>(tile);
+    const float4 *P1 = P0 + S / 2;
+    const float4 *V0 = P1 + S / 2;
+    const float2 *V1 = reinterpret_cast<const float2 *>(V0 + S / 2);
+    const float2 *L2 = reinterpret_cast<const float2 *>(lo);      // 3 planes of S/2 pairs
 #pragma unroll 2
-    for (int j = 0; j < S; ++j) {
-        const int k = j >> 1, h = j & 1;
-        const float x = tile[4 * k + h], y = tile[4 * k + 2 + h];
-        const float z = tile[2 * S + 4 * k + h];
-        const float bx = tile[4 * S + 4 * k + h], by = tile[4 * S + 4 * k + 2 + h];
-        const float bz = tile[6 * S + 2 * k + h];
-        const float xl = lo[j], yl = lo[S + j], zl = lo[2 * S + j];
-        const int64_t jg = jbase + j;
+    for (int k = 0; k < S / 2; ++k) {
+        const float4 p0 = P0[k], p1 = P1[k], v0 = V0[k];
+        const float2 bz = V1[k];
+        const float2 bx = make_float2(v0.x, v0.y), by = make_float2(v0.z, v0.w);
+        const float2 lx = L2[k], ly = L2[S / 2 + k], lz = L2[S + k];
 #pragma unroll
         for (int q = 0; q < KT; ++q) {
-            const float dx = (x - tx[q][0]) + (xl - tl[q][0]);
-            const float dy = (y - tx[q][1]) + (yl - tl[q][1]);
-            const float dz = (z - tx[q][2]) + (zl - tl[q][2]);
-            const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-            if (r2 < 4.0f * h2 && tk[q] >= 0 && jg != tk[q] && record(q, jg)) continue;
-            const float ri = rsqrt_sfu(r2);
-            const float ri2 = ri * ri;
-            float f = ri * ri2;
-            float gp = f * ri2;
-            if (r2 < h2) {
-                float F, Gp, P;
-                spline_kernel<float>(sqrtf(r2) * hinv, F, Gp, P);
-                f = F * hinv3;
-                gp = Gp * hinv5;
-                if (jg == tk[q]) {
-                    f = 0.0f;
-                    gp = 0.0f;
-                }
+            const float2 dx = __fadd2_rn(__fadd2_rn(make_float2(p0.x, p0.y), make_float2(-tx[q][0], -tx[q][0])),
+                                         __fadd2_rn(lx, make_float2(-tl[q][0], -tl[q][0])));
+            const float2 dy = __fadd2_rn(__fadd2_rn(make_float2(p0.z, p0.w), make_float2(-tx[q][1], -tx[q][1])),
+                                         __fadd2_rn(ly, make_float2(-tl[q][1], -tl[q][1])));
+            const float2 dz = __fadd2_rn(__fadd2_rn(make_float2(p1.x, p1.y), make_float2(-tx[q][2], -tx[q][2])),
+                                         __fadd2_rn(lz, make_float2(-tl[q][2], -tl[q][2])));
+            const float2 r2 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, __fmul2_rn(dz, dz)));
+            const float2 ri = make_float2(rsqrt_sfu(r2.x), rsqrt_sfu(r2.y));
+            const float2 ri2 = __fmul2_rn(ri, ri);
+            float2 f = __fmul2_rn(ri, ri2);
+            float2 gp = __fmul2_rn(f, ri2);
+            if (fminf(r2.x, r2.y) < 4.0f * h2) {
+                // a recorded pair leaves the FP32 sums: its terms become 0
+                auto special = [&](float r2s, int64_t jg, float &fs, float &gs) {
+                    if (!(r2s < 4.0f * h2)) return;
+                    if (tk[q] >= 0 && jg != tk[q] && record(q, jg)) {
+                        fs = gs = 0.0f;
+                    } else if (r2s < h2) {
+                        float F, Gp, P;
+                        spline_kernel<float>(sqrtf(r2s) * hinv, F, Gp, P);
+                        fs = F * hinv3;
+                        gs = Gp * hinv5;
+                        if (jg == tk[q]) fs = gs = 0.0f;
+                    }
+                };
+                special(r2.x, jbase + 2 * k, f.x, gp.x);
+                special(r2.y, jbase + 2 * k + 1, f.y, gp.y);
             }
-            const float da = fmaf(dx, bx, fmaf(dy, by, dz * bz));
-            acc[q][X10 + 0].x = fmaf(f, bx, acc[q][X10 + 0].x);
-            acc[q][X10 + 1].x = fmaf(f, by, acc[q][X10 + 1].x);
-            acc[q][X10 + 2].x = fmaf(f, bz, acc[q][X10 + 2].x);
-            const float gd = gp * da;
-            acc[q][X20 + 0].x = fmaf(gd, dx, acc[q][X20 + 0].x);
-            acc[q][X20 + 1].x = fmaf(gd, dy, acc[q][X20 + 1].x);
-            acc[q][X20 + 2].x = fmaf(gd, dz, acc[q][X20 + 2].x);
-            acc[q][MBS].x = fmaf(f, da, acc[q][MBS].x);
+            const float2 da = __ffma2_rn(dx, bx, __ffma2_rn(dy, by, __fmul2_rn(dz, bz)));
+            const float2 gd = __fmul2_rn(gp, da);
+            auto add = [&](float fs, float px, float py, float pz, float ux, float uy, float uz, float ds,
+                           float gs) {
+                acc[q][X10 + 0].x = fmaf(fs, ux, acc[q][X10 + 0].x);
+                acc[q][X10 + 1].x = fmaf(fs, uy, acc[q][X10 + 1].x);
+                acc[q][X10 + 2].x = fmaf(fs, uz, acc[q][X10 + 2].x);
+                acc[q][X20 + 0].x = fmaf(gs, px, acc[q][X20 + 0].x);
+                acc[q][X20 + 1].x = fmaf(gs, py, acc[q][X20 + 1].x);
+                acc[q][X20 + 2].x = fmaf(gs, pz, acc[q][X20 + 2].x);
+                acc[q][MBS].x = fmaf(fs, ds, acc[q][MBS].x);
+            };
+            add(f.x, dx.x, dy.x, dz.x, bx.x, by.x, bz.x, da.x, gd.x);
+            add(f.y, dx.y, dy.y, dz.y, bx.y, by.y, bz.y, da.y, gd.y);
         }
     }
 }
