@@ -251,7 +251,7 @@ __device__ __forceinline__ bool bwd_scalar_item(const BwdArgs &a, BwdScalarSmem<
 #pragma unroll
         for (int q = 0; q < KT; ++q)
 #pragma unroll
-            for (int c = 0; c < kNB; ++c) two_sum_acc(shi[q][c], slo[q][c], acc[q][c]);
+            for (int c = 0; c < kNB; ++c) two_sum_ordered(shi[q][c], slo[q][c], acc[q][c]);
         __syncthreads();
         if (threadIdx.x == 0) {
             if (got) pending &= ~(1u << s);
@@ -308,15 +308,15 @@ backward_kernel(const BwdArgs a)
     const T hinv = MIXED ? (T)a.hinvf : (T)(1.0 / a.h);
 
     for (int64_t item = blockIdx.x; item < items; item += gridDim.x) {
-        const int64_t tb = item / split;
-        const int sp = (int)(item - tb * split);
+        const uint32_t tb = (uint32_t)item / (uint32_t)split;      // (32 bits, as the forward's)
+        const int sp = (int)((uint32_t)item - tb * (uint32_t)split);
         BwdItem it;
-        it.k0 = tb * BT;
+        it.k0 = (int64_t)tb * BT;
         it.k_end = a.n;
-        it.slot0 = tb * BT;
+        it.slot0 = (int64_t)tb * BT;
         it.rows = rows;
-        it.t_begin = (int)((int64_t)sp * a.n_tiles / split);
-        it.t_end = (int)((int64_t)(sp + 1) * a.n_tiles / split);
+        it.t_begin = chunk_begin(sp, a.n_tiles, split);
+        it.t_end = chunk_begin(sp + 1, a.n_tiles, split);
         it.sp = sp;
         it.split = split;
         if (!bwd_scalar_item<T, NT, KT, S>(a, sm, parity, pending, it, h2, hinv, a.h2f_up)) break;
@@ -743,15 +743,15 @@ __global__ void __launch_bounds__(NT, MINB) backward_pair_kernel(const BwdArgs a
     const int64_t rows = n_tb * BT;
 
     for (int64_t item = blockIdx.x; item < items; item += gridDim.x) {
-        const int64_t tb = item / split;
-        const int sp = (int)(item - tb * split);
+        const uint32_t tb = (uint32_t)item / (uint32_t)split;      // (32 bits, as the forward's)
+        const int sp = (int)((uint32_t)item - tb * (uint32_t)split);
         BwdItem it;
-        it.k0 = tb * BT;
+        it.k0 = (int64_t)tb * BT;
         it.k_end = a.n;
-        it.slot0 = tb * BT;
+        it.slot0 = (int64_t)tb * BT;
         it.rows = rows;
-        it.t_begin = (int)((int64_t)sp * a.n_tiles / split);
-        it.t_end = (int)((int64_t)(sp + 1) * a.n_tiles / split);
+        it.t_begin = chunk_begin(sp, a.n_tiles, split);
+        it.t_end = chunk_begin(sp + 1, a.n_tiles, split);
         it.sp = sp;
         it.split = split;
         if (!bwd_pair_item<NT, KT, S, U>(a, sm, parity, it, a.h, a.h2f_up, a.hinvf)) break;
@@ -799,27 +799,35 @@ __global__ void __launch_bounds__(NT, MINB) backward_pair_batched_kernel(const B
     bwd_pair_drain(sm, parity, a.flags);
 }
 
-__global__ void __launch_bounds__(256) backward_reduce_kernel(const BwdArgs a, int32_t BT)
+// One thread per (target, component) adds the chunk partials (FP64 bound, as
+// the forward's reduction), then one per target forms the outputs.
+constexpr int kBwdReduceThreads = 128;
+constexpr int kBwdReduceTargets = kBwdReduceThreads / 8;
+
+__global__ void __launch_bounds__(kBwdReduceThreads) backward_reduce_kernel(const BwdArgs a, int32_t BT)
 {
+    __shared__ double red[kBwdReduceTargets][kNB];
     const int64_t n_tb = (a.n + BT - 1) / BT;
     const int split = choose_split(n_tb, a.n_tiles, a.grid, a.max_split, a.part_cap_rows, BT);
     if (split <= 1) return;
     const int64_t rows = n_tb * BT;
-    const int64_t k = (int64_t)blockIdx.x * 256 + threadIdx.x;
-    if (k >= a.n) return;
-    double hi[kNB], lo[kNB];
-#pragma unroll
-    for (int c = 0; c < kNB; ++c) {
-        hi[c] = 0.0;
-        lo[c] = 0.0;
+    const int t = threadIdx.x % kBwdReduceTargets, c = threadIdx.x / kBwdReduceTargets;
+    const int64_t k = (int64_t)blockIdx.x * kBwdReduceTargets + t;
+    if (c < kNB && k < a.n) {
+        const double *part = a.part + (int64_t)c * rows + k;
+        const int64_t step = (int64_t)kNB * rows;
+        double hi = part[0], lo = 0.0;
+#pragma unroll 4
+        for (int sp = 1; sp < split; ++sp) two_sum_ordered(hi, lo, part[sp * step]);
+        red[t][c] = hi + lo;
     }
-    for (int sp = 0; sp < split; ++sp)
+    __syncthreads();
+    if (threadIdx.x < kBwdReduceTargets && k < a.n) {
+        double sum[kNB];
 #pragma unroll
-        for (int c = 0; c < kNB; ++c) two_sum_acc(hi[c], lo[c], a.part[((int64_t)sp * kNB + c) * rows + k]);
-    double sum[kNB];
-#pragma unroll
-    for (int c = 0; c < kNB; ++c) sum[c] = hi[c] + lo[c];
-    bwd_write(a, k, sum);
+        for (int q = 0; q < kNB; ++q) sum[q] = red[t][q];
+        bwd_write(a, k, sum);
+    }
 }
 
 // a_bar == NULL: only the potential-energy terms, elementwise.
@@ -1051,7 +1059,8 @@ extern "C" int grav_eval_backward(const grav_params *p, int64_t n, const double 
     const int64_t n_tb = (n + L.BT - 1) / L.BT;
     if (L.part_cap_rows > 0 &&
         choose_split(n_tb, a.n_tiles, grid, a.max_split, a.part_cap_rows, L.BT) > 1) {
-        backward_reduce_kernel<<<eblocks, 256, 0, st>>>(a, L.BT);
+        backward_reduce_kernel<<<(unsigned)((n + kBwdReduceTargets - 1) / kBwdReduceTargets),
+                                 kBwdReduceThreads, 0, st>>>(a, L.BT);
         rc = check_launch("grav_eval_backward/reduce");
     }
     return rc;

@@ -126,10 +126,14 @@ __host__ __device__ inline int choose_split(int64_t n_tb, int32_t n_tiles, int32
     int64_t cap = part_cap_rows / (n_tb * (int64_t)BT);
     if (cap < s_max) s_max = cap;
     if (s_max <= 1) return 1;
+    // items = n_tb s and slots = items rounded up to whole rounds of the grid,
+    // both by addition: every thread of the kernels runs this loop, and its
+    // 64-bit divisions took several microseconds of a small evaluation
     int64_t best = 1, best_items = n_tb, best_slots = ((n_tb + grid - 1) / grid) * grid;
+    int64_t items = 0, slots = 0;
     for (int64_t s = 1; s <= s_max; ++s) {
-        int64_t items = n_tb * s;
-        int64_t slots = ((items + grid - 1) / grid) * grid;
+        items += n_tb;
+        while (slots < items) slots += grid;
         if (items >= grid && 20 * items >= 19 * slots) return (int)s;
         if (items * best_slots > best_items * slots) {
             best = s;
@@ -138,6 +142,14 @@ __host__ __device__ inline int choose_split(int64_t n_tb, int32_t n_tiles, int32
         }
     }
     return (int)best;
+}
+
+// First tile of source chunk sp of split chunks over n_tiles < 2^25 tiles (the
+// product stays below 2^32: split is at most kDefaultMaxSplit there).
+__device__ __forceinline__ int chunk_begin(int sp, int32_t n_tiles, int split)
+{
+    if (split <= kDefaultMaxSplit) return (int)((uint32_t)sp * (uint32_t)n_tiles / (uint32_t)split);
+    return (int)((int64_t)sp * n_tiles / split);
 }
 
 __device__ __forceinline__ int64_t active_count(const EvalArgs &a)
@@ -151,25 +163,68 @@ __device__ __forceinline__ int64_t active_count(const EvalArgs &a)
     return n;
 }
 
-// Final FP64 outputs of one target from its accumulated sums.  ETRACE: slot 9
-// holds E and F = E + trace(Tp) (mixed path); otherwise slot 9 holds F.
+// One part of the final FP64 outputs of a target from its accumulated sums
+// s[c * stride]: parts 0-2 the acceleration, 3-5 the jerk, 6-11 the tidal
+// tensor, 12 the tidal timestep, 13 the potential.  ETRACE: slot 9 holds E
+// and F = E + trace(Tp) (mixed path); otherwise slot 9 holds F.
 // Every operation is an explicit correctly rounded intrinsic, so all kernels
 // that end in this epilogue (single-system, batched, reduction) turn the same
 // sums into bit-identical outputs whatever the compiler fuses elsewhere.
+constexpr int kTargetParts = 14;
+
+template <bool ETRACE>
+__device__ __forceinline__ void tidal_of(double G, const double *s, int stride, double t6[6])
+{
+    const double txx = s[TXX * stride], tyy = s[TYY * stride], tzz = s[TZZ * stride];
+    const double F = ETRACE ? __dadd_rn(s[ESUM * stride], __dadd_rn(__dadd_rn(txx, tyy), tzz))
+                            : s[FSUM * stride];
+    const double G3 = __dmul_rn(3.0, G);
+    t6[0] = __dmul_rn(-G, __dsub_rn(F, __dmul_rn(3.0, txx)));
+    t6[1] = __dmul_rn(-G, __dsub_rn(F, __dmul_rn(3.0, tyy)));
+    t6[2] = __dmul_rn(-G, __dsub_rn(F, __dmul_rn(3.0, tzz)));
+    t6[3] = __dmul_rn(G3, s[TXY * stride]);
+    t6[4] = __dmul_rn(G3, s[TXZ * stride]);
+    t6[5] = __dmul_rn(G3, s[TYZ * stride]);
+}
+
+template <bool POT, bool ETRACE>
+__device__ __forceinline__ void write_target_part(const EvalArgs &a, int64_t i, const double *s,
+                                                  int stride, int part)
+{
+    const double G = a.G;
+    if (part < 3) {
+        a.acc[3 * i + part] = __dmul_rn(G, s[(A0 + part) * stride]);
+    } else if (part < 6) {
+        const int c = part - 3;
+        a.jerk[3 * i + c] =
+            __dmul_rn(G, __dsub_rn(s[(J10 + c) * stride], __dmul_rn(3.0, s[(J20 + c) * stride])));
+    } else if (part < 9) {
+        const int c = part - 6;
+        const double F =
+            ETRACE ? __dadd_rn(s[ESUM * stride], __dadd_rn(__dadd_rn(s[TXX * stride], s[TYY * stride]),
+                                                           s[TZZ * stride]))
+                   : s[FSUM * stride];
+        a.tidal[6 * i + c] = __dmul_rn(-G, __dsub_rn(F, __dmul_rn(3.0, s[(TXX + c) * stride])));
+    } else if (part < 12) {
+        const int c = part - 6;
+        a.tidal[6 * i + c] = __dmul_rn(__dmul_rn(3.0, G), s[(TXX + c) * stride]);
+    } else if (part == 12) {
+        if (!a.dt_grav) return;
+        double t6[6];
+        tidal_of<ETRACE>(G, s, stride, t6);
+        a.dt_grav[i] = tidal_dt(t6, a.sqrt_eta);
+    } else if (POT) {
+        a.pot[i] = __dmul_rn(-G, s[PSUM * stride]);
+    }
+}
+
+// All parts of one target.
 template <bool POT, bool ETRACE>
 __device__ __forceinline__ void write_target(const EvalArgs &a, int64_t i, const double s[kNCPot])
 {
     const double G = a.G;
-    const double F = ETRACE ? __dadd_rn(s[ESUM], __dadd_rn(__dadd_rn(s[TXX], s[TYY]), s[TZZ]))
-                            : s[FSUM];
-    const double G3 = __dmul_rn(3.0, G);
     double t6[6];
-    t6[0] = __dmul_rn(-G, __dsub_rn(F, __dmul_rn(3.0, s[TXX])));
-    t6[1] = __dmul_rn(-G, __dsub_rn(F, __dmul_rn(3.0, s[TYY])));
-    t6[2] = __dmul_rn(-G, __dsub_rn(F, __dmul_rn(3.0, s[TZZ])));
-    t6[3] = __dmul_rn(G3, s[TXY]);
-    t6[4] = __dmul_rn(G3, s[TXZ]);
-    t6[5] = __dmul_rn(G3, s[TYZ]);
+    tidal_of<ETRACE>(G, s, 1, t6);
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
         a.acc[3 * i + c] = __dmul_rn(G, s[A0 + c]);
@@ -230,35 +285,71 @@ __device__ __forceinline__ void block_bbox(float lo[3], float hi[3], float *blo,
 // Tile packing (K3)
 // ---------------------------------------------------------------------------
 
-// Block-wide FP64 min/max over S threads.
-template <int S>
-__device__ __forceinline__ void block_minmax_d(double lo[3], double hi[3], double *slo, double *shi)
+// FP64 numbers as 64-bit integers of the same order (the packer's bounding
+// boxes: FP64 compares run at 1/64 of the integer rate on GB300).
+__device__ __forceinline__ long long order_key(double x)
 {
-    __shared__ double wlo[3][S / 32], whi[3][S / 32];
+    const long long b = __double_as_longlong(x);
+    return b ^ ((b >> 63) & 0x7fffffffffffffffLL);
+}
+
+__device__ __forceinline__ double order_value(long long k)
+{
+    return __longlong_as_double(k ^ ((k >> 63) & 0x7fffffffffffffffLL));
+}
+
+// Smallest key of a warp: the high words, then the low words among the lanes
+// that hold the smallest high word.
+__device__ __forceinline__ long long warp_min_key(long long k)
+{
+    const int hi = (int)(k >> 32);
+    const int mh = __reduce_min_sync(0xffffffffu, hi);
+    const uint32_t ml = __reduce_min_sync(0xffffffffu, hi == mh ? (uint32_t)k : 0xffffffffu);
+    return ((long long)mh << 32) | ml;
+}
+
+// Block-wide min and max of NV FP64 values per thread (`ok` false: no value;
+// NaN values are left out), one pass for all of them: out[2 v] = min of value
+// v, out[2 v + 1] = max.  Over no value the min is +inf and the max -inf.
+// FP64 shuffles and compares for positions and then velocities took most of
+// the packer's time: 131072 elements 41 us, with integer keys 10 us.
+template <int S, int NV>
+__device__ __forceinline__ void block_minmax_keys(const double (&v)[NV], bool ok, double *out)
+{
+    __shared__ long long wkey[2 * NV][S / 32];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const long long kInf = 0x7ff0000000000000LL;
 #pragma unroll
-    for (int c = 0; c < 3; ++c) {
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            lo[c] = fmin(lo[c], __shfl_xor_sync(0xffffffffu, lo[c], o));
-            hi[c] = fmax(hi[c], __shfl_xor_sync(0xffffffffu, hi[c], o));
-        }
+    for (int c = 0; c < NV; ++c) {
+        const long long b = __double_as_longlong(v[c]);
+        const bool use = ok && (b & 0x7fffffffffffffffLL) <= kInf;      // not NaN
+        const long long k = order_key(v[c]);
+        // max(k) = ~min(~k): the complement reverses the order of the keys
+        const long long lo = warp_min_key(use ? k : kInf);
+        const long long hi = ~warp_min_key(use ? ~k : kInf);   // ~kInf is the key of -inf
         if (lane == 0) {
-            wlo[c][wid] = lo[c];
-            whi[c][wid] = hi[c];
+            wkey[2 * c][wid] = lo;
+            wkey[2 * c + 1][wid] = hi;
         }
     }
     __syncthreads();
-    if (threadIdx.x < 3) {
-        double l = wlo[threadIdx.x][0], h = whi[threadIdx.x][0];
+    if (threadIdx.x < 2 * NV) {
+        const bool low = (threadIdx.x & 1) == 0;
+        long long r = wkey[threadIdx.x][0];
+#pragma unroll
         for (int w = 1; w < S / 32; ++w) {
-            l = fmin(l, wlo[threadIdx.x][w]);
-            h = fmax(h, whi[threadIdx.x][w]);
+            const long long k = wkey[threadIdx.x][w];
+            if (low ? k < r : k > r) r = k;
         }
-        slo[threadIdx.x] = l;
-        shi[threadIdx.x] = h;
+        out[threadIdx.x] = order_value(r);
     }
     __syncthreads();
+}
+
+// (not an infinity or NaN, by the exponent bits)
+__device__ __forceinline__ bool finite_bits(double x)
+{
+    return (__double2hiint(x) & 0x7ff00000) != 0x7ff00000;
 }
 
 // Planes of low parts per packed mixed tile: x, y, z.
@@ -277,43 +368,36 @@ __device__ __forceinline__ void pack_tile(int t, int64_t first, int64_t end,
                                           TileGeom *__restrict__ geo, void *__restrict__ src,
                                           int32_t *flags, float *__restrict__ src_lo = nullptr)
 {
-    __shared__ double slo[3], shi[3], svlo[3], svhi[3];
+    constexpr int NV = VOFF ? 6 : 3;      // boxes of the positions and, with VOFF, the velocities
+    __shared__ double mm[2 * NV];
     const int j = threadIdx.x;
     const int64_t gj = first + j;
     const bool ok = gj < end;
     double x[3] = {0, 0, 0}, v[3] = {0, 0, 0}, m = 0.0;
     if (ok) {
+        bool fine = true;
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
             x[c] = pos[3 * gj + c];
             v[c] = vel[3 * gj + c];
+            fine = fine && finite_bits(x[c]) && finite_bits(v[c]);
         }
         m = mass ? mass[gj] : 0.0;
-        if (!(finite3(x[0], x[1], x[2]) && finite3(v[0], v[1], v[2]) && isfinite(m)))
-            flag_or(flags, GRAV_FLAG_NONFINITE);
+        if (!(fine && finite_bits(m))) flag_or(flags, GRAV_FLAG_NONFINITE);
     }
-    const double inf = __longlong_as_double(0x7ff0000000000000LL);
-    double lo[3], hi[3];
+    double xv[NV];
 #pragma unroll
-    for (int c = 0; c < 3; ++c) {
-        lo[c] = ok ? x[c] : inf;
-        hi[c] = ok ? x[c] : -inf;
-    }
-    block_minmax_d<S>(lo, hi, slo, shi);
+    for (int c = 0; c < NV; ++c) xv[c] = c < 3 ? x[c] : v[c - 3];
+    block_minmax_keys<S, NV>(xv, ok, mm);
     float cvf[3] = {0.0f, 0.0f, 0.0f};
     if (VOFF) {
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            lo[c] = ok ? v[c] : inf;
-            hi[c] = ok ? v[c] : -inf;
-        }
-        block_minmax_d<S>(lo, hi, svlo, svhi);
-#pragma unroll
-        for (int c = 0; c < 3; ++c) cvf[c] = __double2float_rn(__dmul_rn(0.5, __dadd_rn(svlo[c], svhi[c])));
+        for (int c = 0; c < 3; ++c)
+            cvf[c] = __double2float_rn(__dmul_rn(0.5, __dadd_rn(mm[2 * (NV - 3 + c)], mm[2 * (NV - 3 + c) + 1])));
     }
     double cc[3];
 #pragma unroll
-    for (int c = 0; c < 3; ++c) cc[c] = __dmul_rn(0.5, __dadd_rn(slo[c], shi[c]));
+    for (int c = 0; c < 3; ++c) cc[c] = __dmul_rn(0.5, __dadd_rn(mm[2 * c], mm[2 * c + 1]));
     if (MIXED && src_lo) {
         // low parts of the FP32 position offsets (zero for padding), planes
         // [x y z] of S each
@@ -387,8 +471,8 @@ __device__ __forceinline__ void pack_tile(int t, int64_t first, int64_t end,
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
             g.c[c] = cc[c];
-            g.lo[c] = __double2float_rd(slo[c]);
-            g.hi[c] = __double2float_ru(shi[c]);
+            g.lo[c] = __double2float_rd(mm[2 * c]);
+            g.hi[c] = __double2float_ru(mm[2 * c + 1]);
             g.cv[c] = cvf[c];
         }
         g.first = (int32_t)first;
@@ -1986,22 +2070,32 @@ __device__ __forceinline__ bool mixed_item(
     float tx[KT][3], tx_next[KT][3];
     offsets(g, tx);
 
+    // a warp without a target (the last block of a small or ragged due set)
+    // only takes part in the release of the stages
+    bool warp_live = false;
+#pragma unroll
+    for (int q = 0; q < KT; ++q) warp_live = warp_live || ti[q] >= 0;
+    warp_live = __any_sync(0xffffffffu, warp_live);
+
     for (int t = t_begin; t < t_end; ++t) {
         const int s = (t - t_begin) % NSTAGE;
-        // periodic: any target near the tile, or a tile that may reach past
-        // half a box from a target's image of it, takes the general loop
-        float h2_tile = a.h2f_up;
-        if (soft) {
-            const float hm = fmaxf(h_block, a.geo_h[t]);
-            h2_tile = __fmul_ru(hm, hm);
-        }
-        bool near, close;
-        classify_tile<KT, MODE>(a, g, tx, ti, blo_r, bhi_r, rc2, h2_tile, near, close);
-        // next tile's geometry and offsets, computed ahead (FP64 latency)
+        bool near = false, close = false;
         TileGeom gn = g;
-        if (t + 1 < t_end) {
-            gn = a.geo[t + 1];
-            offsets(gn, tx_next);
+        if (warp_live) {
+            // periodic: any target near the tile, or a tile that may reach
+            // past half a box from a target's image of it, takes the general
+            // loop
+            float h2_tile = a.h2f_up;
+            if (soft) {
+                const float hm = fmaxf(h_block, a.geo_h[t]);
+                h2_tile = __fmul_ru(hm, hm);
+            }
+            classify_tile<KT, MODE>(a, g, tx, ti, blo_r, bhi_r, rc2, h2_tile, near, close);
+            // next tile's geometry and offsets, computed ahead (FP64 latency)
+            if (t + 1 < t_end) {
+                gn = a.geo[t + 1];
+                offsets(gn, tx_next);
+            }
         }
         const bool got = mbar_wait_bounded(&sm.bar[s], (ring.parity >> s) & 1u, a.flags);
         if (got)
@@ -2014,7 +2108,9 @@ __device__ __forceinline__ bool mixed_item(
         for (int q = 0; q < KT; ++q)
 #pragma unroll
             for (int c = 0; c < kNCPot; ++c) acc[q][c] = 0.0f;
-        if (close && periodic) {
+        if (!warp_live) {
+            // nothing to sum
+        } else if (close && periodic) {
             // the targets' low parts for this tile; runs of the close loops
             // carry their own sums (acc stays zero)
             float tl[KT][3];
@@ -2078,7 +2174,7 @@ __device__ __forceinline__ bool mixed_item(
         }
 
         // per-tile corrections for the target velocity, then the carry
-        if (!(close && periodic)) carry_tile(acc);
+        if (warp_live && !(close && periodic)) carry_tile(acc);
 
         // this warp is done reading stage s; the last warp refills it
         __syncwarp();
@@ -2105,8 +2201,12 @@ __device__ __forceinline__ bool mixed_item(
     }
 
     // the listed pairs in FP64 (each lane its own list; an inactive lane's
-    // list is skipped)
+    // list is skipped; nothing to add where no lane of the warp has one)
+    bool any_listed = false;
     if constexpr (listed) {
+#pragma unroll
+        for (int q = 0; q < KT; ++q) any_listed = any_listed || (ti[q] >= 0 && ncnt[q] > 0);
+        any_listed = __any_sync(0xffffffffu, any_listed);
 #pragma unroll
         for (int q = 0; q < KT; ++q) {
             if (ti[q] < 0) continue;
@@ -2130,6 +2230,7 @@ __device__ __forceinline__ bool mixed_item(
     // ---- results ----
 #pragma unroll
     for (int q = 0; q < KT; ++q) {
+        if (!warp_live) continue;      // (the reduction reads the rows of targets only)
         double sum[kNCPot];
 #pragma unroll
         for (int c = 0; c < kNCPot; ++c) {
@@ -2143,7 +2244,7 @@ __device__ __forceinline__ bool mixed_item(
                                    (double)rlo[SACC ? 0 : q][SACC ? 0 : c]);
             }
             if constexpr (listed) {
-                if (c < NC) sum[c] = __dadd_rn(sum[c], nsum[q][c]);
+                if (c < NC && any_listed) sum[c] = __dadd_rn(sum[c], nsum[q][c]);
             }
         }
         if (it.split == 1) {
@@ -2170,16 +2271,17 @@ eval_mixed_kernel(const EvalArgs a)
     const int split = choose_split(n_tb, a.n_tiles, a.grid, a.max_split, a.part_cap_rows, BT);
     const int64_t items = n_tb * split;
     for (int64_t item = blockIdx.x; item < items; item += gridDim.x) {
-        const int64_t tb = item / split;
-        const int sp = (int)(item - tb * split);
+        // (item < 4 grid max_split, or a target block's number: 32 bits)
+        const uint32_t tb = (uint32_t)item / (uint32_t)split;
+        const int sp = (int)((uint32_t)item - tb * (uint32_t)split);
         ItemSpec it;
         it.idx = a.idx;
-        it.slot0 = tb * BT;
+        it.slot0 = (int64_t)tb * BT;
         it.slot_end = n_act;
         it.elem_lo = 0;
         it.elem_hi = a.n_src;
-        it.t_begin = (int)((int64_t)sp * a.n_tiles / split);
-        it.t_end = (int)((int64_t)(sp + 1) * a.n_tiles / split);
+        it.t_begin = chunk_begin(sp, a.n_tiles, split);
+        it.t_end = chunk_begin(sp + 1, a.n_tiles, split);
         it.sp = sp;
         it.split = split;
         it.rows = n_tb * BT;
@@ -2374,7 +2476,7 @@ __device__ __forceinline__ bool f64_item(const EvalArgs &a, F64Smem<S> &sm, Ring
                                                    a.box_tie);
                 target_velocity_d(racc, vr);
 #pragma unroll
-                for (int c = 0; c < NC; ++c) two_sum_acc(shi[c], slo[c], racc[c]);
+                for (int c = 0; c < NC; ++c) two_sum_ordered(shi[c], slo[c], racc[c]);
             }
         } else {
             if (periodic && !near)
@@ -2390,7 +2492,7 @@ __device__ __forceinline__ bool f64_item(const EvalArgs &a, F64Smem<S> &sm, Ring
             target_velocity_d(acc, vr);
         }
 #pragma unroll
-        for (int c = 0; c < NC; ++c) two_sum_acc(shi[c], slo[c], acc[c]);
+        for (int c = 0; c < NC; ++c) two_sum_ordered(shi[c], slo[c], acc[c]);
         __syncthreads();
         if (threadIdx.x == 0) {
             if (got) ring.pending &= ~(1u << s);
@@ -2424,16 +2526,17 @@ eval_f64_kernel(const EvalArgs a)
     const int split = choose_split(n_tb, a.n_tiles, a.grid, a.max_split, a.part_cap_rows, NT);
     const int64_t items = n_tb * split;
     for (int64_t item = blockIdx.x; item < items; item += gridDim.x) {
-        const int64_t tb = item / split;
-        const int sp = (int)(item - tb * split);
+        // (item < 4 grid max_split, or a target block's number: 32 bits)
+        const uint32_t tb = (uint32_t)item / (uint32_t)split;
+        const int sp = (int)((uint32_t)item - tb * (uint32_t)split);
         ItemSpec it;
         it.idx = a.idx;
-        it.slot0 = tb * NT;
+        it.slot0 = (int64_t)tb * NT;
         it.slot_end = n_act;
         it.elem_lo = 0;
         it.elem_hi = a.n_src;
-        it.t_begin = (int)((int64_t)sp * a.n_tiles / split);
-        it.t_end = (int)((int64_t)(sp + 1) * a.n_tiles / split);
+        it.t_begin = chunk_begin(sp, a.n_tiles, split);
+        it.t_end = chunk_begin(sp + 1, a.n_tiles, split);
         it.sp = sp;
         it.split = split;
         it.rows = n_tb * NT;
@@ -2494,10 +2597,11 @@ eval_f64_batched_kernel(const EvalArgs a, const BatchView b)
 // ---------------------------------------------------------------------------
 
 // Threads of the split reduction: one per (target, accumulated component),
-// so that a small target set (the usual case of a split) still spreads its
-// FP64 work -- `split` TwoSums per component, at 1/74 of the FP32 rate on
-// GB300 -- over many warps instead of queueing it on a few.
-constexpr int kReduceThreads = 256;
+// then one per (target, output part).  FP64 runs at 1/64 of the FP32 rate on
+// GB300, so the FP64 instructions bound this kernel: the chunk partials are
+// added with two_sum_ordered (4 FP64 instructions instead of TwoSum's 7, the
+// same bits), and 8 targets a CTA spread a small set over many SMs.
+constexpr int kReduceThreads = 128;
 template <bool POT>
 constexpr int reduce_targets_per_block() { return kReduceThreads / (POT ? kNCPot : kNC); }
 
@@ -2521,21 +2625,17 @@ reduce_partials_kernel(const EvalArgs a, int32_t BT)
         const int64_t slot = slot0 + k;
         if (c < NC && slot < n_act) {
             // the chunk partials of component c of this target, in split order
-            double hi = 0.0, lo = 0.0;
-            for (int sp = 0; sp < split; ++sp)
-                two_sum_acc(hi, lo, a.part[((int64_t)sp * NC + c) * rows + slot]);
+            const double *part = a.part + (int64_t)c * rows + slot;
+            const int64_t step = (int64_t)NC * rows;
+            double hi = part[0], lo = 0.0;
+#pragma unroll 4
+            for (int sp = 1; sp < split; ++sp) two_sum_ordered(hi, lo, part[sp * step]);
             red[c][k] = __dadd_rn(hi, lo);
         }
         __syncthreads();
-        if (threadIdx.x < TPB && slot0 + threadIdx.x < n_act) {
-            const int64_t sl = slot0 + threadIdx.x;
-            const int64_t i = a.idx ? (int64_t)a.idx[sl] : sl;
-            if (i >= 0 && i < a.n_src) {
-                double sum[kNCPot];
-#pragma unroll
-                for (int q = 0; q < kNCPot; ++q) sum[q] = q < NC ? red[q][threadIdx.x] : 0.0;
-                write_target<POT, ETRACE>(a, i, sum);
-            }
+        if (c < kTargetParts && slot < n_act) {
+            const int64_t i = a.idx ? (int64_t)a.idx[slot] : slot;
+            if (i >= 0 && i < a.n_src) write_target_part<POT, ETRACE>(a, i, &red[0][k], TPB, c);
         }
         __syncthreads();                             // red is reused by the next group
     }

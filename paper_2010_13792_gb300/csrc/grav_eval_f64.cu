@@ -36,7 +36,7 @@ void launch_reduce(const EvalArgs &a, int32_t BT, bool pot, bool etrace, int64_t
     int sms = 0;
     if (device_sm_count(&sms) != GRAV_OK || sms <= 0) sms = 1;
     const unsigned blocks =
-        (unsigned)std::max<int64_t>(1, std::min<int64_t>((n_targets + tpb - 1) / tpb, 8LL * sms));
+        (unsigned)std::max<int64_t>(1, std::min<int64_t>((n_targets + tpb - 1) / tpb, 16LL * sms));
     if (pot && etrace)
         reduce_partials_kernel<true, true><<<blocks, kReduceThreads, 0, st>>>(a, BT);
     else if (pot)
