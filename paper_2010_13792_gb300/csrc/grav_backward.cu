@@ -326,7 +326,7 @@ backward_kernel(const BwdArgs a)
 }
 
 // Batched scalar adjoint: the items of all systems from the plan, taken
-// through an atomic ticket; each system's targets against its own tiles
+// from the per-SM queues; each system's targets against its own tiles
 // with its own support h (grav_system.h, or the call's h where it is 0).
 template <int NT, int KT, int S, int MINB>
 __global__ void __launch_bounds__(NT, MINB)
@@ -338,11 +338,14 @@ backward_batched_kernel(const BwdArgs a, const BatchView b)
     uint32_t parity = 0, pending = 0;
     const int64_t total = b.hdr->total_items;
     for (;;) {
-        if (threadIdx.x == 0) sm.ticket = (long long)atomicAdd(&b.hdr->ticket, 1ULL);
+        if (threadIdx.x < 32) {
+            const int64_t tk = take_item(b, total);
+            if (threadIdx.x == 0) sm.ticket = tk;
+        }
         __syncthreads();
         const int64_t ticket = sm.ticket;
         __syncthreads();
-        if (ticket >= total) break;
+        if (ticket < 0) break;
         const int r = item_rank(b, ticket);
         const int s = b.order[r];
         const double h = b.sys[s].h > 0.0 ? b.sys[s].h : a.h;
@@ -761,7 +764,7 @@ __global__ void __launch_bounds__(NT, MINB) backward_pair_kernel(const BwdArgs a
 }
 
 // Batched mixed adjoint: the items of all systems from the plan, taken
-// through an atomic ticket; each system's targets against its own tiles with
+// from the per-SM queues; each system's targets against its own tiles with
 // its own support h (grav_system.h, or the call's h where it is 0).
 template <int NT, int KT, int S, int MINB, int U>
 __global__ void __launch_bounds__(NT, MINB) backward_pair_batched_kernel(const BwdArgs a,
@@ -774,11 +777,14 @@ __global__ void __launch_bounds__(NT, MINB) backward_pair_batched_kernel(const B
     uint32_t parity = 0;
     const int64_t total = b.hdr->total_items;
     for (;;) {
-        if (threadIdx.x == 0) sm.ticket = (long long)atomicAdd(&b.hdr->ticket, 1ULL);
+        if (threadIdx.x < 32) {
+            const int64_t tk = take_item(b, total);
+            if (threadIdx.x == 0) sm.ticket = tk;
+        }
         __syncthreads();
         const int64_t ticket = sm.ticket;
         __syncthreads();
-        if (ticket >= total) break;
+        if (ticket < 0) break;
         const int r = item_rank(b, ticket);
         const int s = b.order[r];
         const double h = b.sys[s].h > 0.0 ? b.sys[s].h : a.h;
@@ -924,7 +930,7 @@ BwdBatchLayout bwd_batch_layout(bool mixed, int32_t n_sys, int64_t n_total)
     L.max_tiles = (n_total + S - 1) / S + n_sys;
     int64_t o = 0;
     L.hdr = o;
-    o += 256;
+    o += kBatchHeaderBytes;
     L.tile_off = o;
     o += round_up(4 * ((int64_t)n_sys + 1), 256);
     L.idx_lo = o;
@@ -1118,7 +1124,8 @@ extern "C" int grav_eval_backward_batched(const grav_params *p, int32_t n_sys,
     b.order = reinterpret_cast<int32_t *>(ws + L.order);
     b.item_off = reinterpret_cast<int64_t *>(ws + L.item_off);
     b.n_sys = n_sys;
-    b.pad = 0;
+    rc = batch_queues(&b.n_queues);
+    if (rc) return rc;
 
     BwdArgs a;
     a.n = n_total;

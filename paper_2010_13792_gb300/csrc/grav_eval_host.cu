@@ -12,10 +12,14 @@ namespace {
 
 // Default tile configurations (measured on 2^20-element clouds, a 2^17
 // Plummer sphere and 64^3 and 96^3 periodic lattices): 768-thread CTAs, one
-// per SM, from 8192 targets; 256-thread CTAs (three per SM) for smaller sets
-// and batched launches, where more CTAs per SM keep the SMs busier through the
-// last round of work items.
+// per SM, from 8192 targets; 256-thread CTAs (three per SM) for smaller sets,
+// where more CTAs per SM keep the SMs busier through the last round of work
+// items.  Batched launches take 128-thread CTAs: their items, which may not
+// be split, are twice as fine (12 systems 944 -> 694 us against 256 threads,
+// 64 systems 1.46 -> 1.37 ms, 256 systems of up to 65536 elements 35.4 ->
+// 34.3 ms).
 constexpr int kDefaultMixed = 11;
+constexpr int kDefaultMixedBatched = 10;
 constexpr int kDefaultMixedLarge = 17;
 constexpr int64_t kLargeTargetSet = 1 << 13;
 constexpr int kDefaultF64 = 0;
@@ -64,6 +68,14 @@ const EvalConfig *resolve(const grav_params *p, int mode, int64_t n_targets, int
     int i = p->tile_config >= 0 ? p->tile_config : default_index(p->precision, mode, n_targets);
     *index = i;
     return &t[i];
+}
+
+const EvalConfig *resolve_batched(const grav_params *p, int *index)
+{
+    if (p->precision != GRAV_MIXED || p->tile_config >= 0) return resolve(p, kModeOpen, 0, index);
+    int n = 0;
+    *index = kDefaultMixedBatched;
+    return &config_table(p->precision, &n)[kDefaultMixedBatched];
 }
 
 // Per source tile for adaptive softening: (1/h_j, zeta_j) in FP32 in tile
@@ -450,7 +462,7 @@ __device__ void cta_exclusive_scan(const TIn *vals, TOut *out, int n)
 
 // The plan of a batched launch (one CTA): per-system tiles and target
 // ranges, the longest-first order of the systems and the work-item offsets;
-// resets the ticket counter.
+// resets the work queues.
 __global__ void __launch_bounds__(kPlanThreads)
 batch_plan_kernel(BatchView b, const int32_t *__restrict__ idx, const int32_t *n_idx_dev,
                   int64_t n_idx_max, int64_t n_total, int32_t S, int32_t BT, double box,
@@ -497,8 +509,8 @@ batch_plan_kernel(BatchView b, const int32_t *__restrict__ idx, const int32_t *n
     if (threadIdx.x == 0) {
         b.hdr->total_items = b.item_off[n];
         b.hdr->total_tiles = b.tile_off[n];
-        b.hdr->ticket = 0ULL;
     }
+    for (int q = threadIdx.x; q < kMaxQueues; q += kPlanThreads) b.hdr->next[q] = 0u;
 }
 
 struct BatchLayout {
@@ -514,7 +526,7 @@ BatchLayout batch_layout(const EvalConfig *c, int32_t n_sys, int64_t n_total)
     L.max_tiles = (n_total + S - 1) / S + n_sys;
     int64_t o = 0;
     L.hdr = o;
-    o += 256;
+    o += kBatchHeaderBytes;
     L.tile_off = o;
     o += round_up(4 * ((int64_t)n_sys + 1), 256);
     L.idx_lo = o;
@@ -563,6 +575,15 @@ int batch_grid_for(const EvalConfig *c, int index, bool periodic, bool pot, int 
 
 }  // namespace
 
+int batch_queues(int32_t *n)
+{
+    int sms = 0;
+    int rc = device_sm_count(&sms);
+    if (rc) return rc;
+    *n = std::min(std::max(sms, 1), kMaxQueues);
+    return GRAV_OK;
+}
+
 int launch_batch_plan(const BatchView &b, const int32_t *idx, const int32_t *n_idx_dev,
                       int64_t n_idx_max, int64_t n_total, int32_t S, int32_t BT, double box,
                       int32_t *flags, cudaStream_t st)
@@ -581,7 +602,7 @@ extern "C" int64_t grav_batched_workspace_bytes(const grav_params *p, int32_t n_
     if (n_sys < 0 || n_sys > GRAV_BATCH_MAX_SYSTEMS || n_total < 0 || n_total > INT32_MAX)
         return fail(GRAV_EINVAL, "grav_batched_workspace_bytes: n_sys or n_total out of range");
     int index = 0;
-    const EvalConfig *c = resolve(p, kModeOpen, 0, &index);
+    const EvalConfig *c = resolve_batched(p, &index);
     return batch_layout(c, n_sys, n_total).total;
 }
 
@@ -606,7 +627,7 @@ extern "C" int grav_eval_batched(const grav_params *p, int32_t n_sys, const grav
     if (!workspace || !aligned(workspace, 256))
         return fail(GRAV_EINVAL, "%s: workspace missing or not 256-byte aligned", who);
     int index = 0;
-    const EvalConfig *c = resolve(p, kModeOpen, 0, &index);
+    const EvalConfig *c = resolve_batched(p, &index);
     const BatchLayout L = batch_layout(c, n_sys, n_total);
     if (workspace_bytes < L.total)
         return fail(GRAV_ENOMEM, "%s: workspace of %lld bytes < %lld", who, (long long)workspace_bytes,
@@ -627,7 +648,8 @@ extern "C" int grav_eval_batched(const grav_params *p, int32_t n_sys, const grav
     b.order = reinterpret_cast<int32_t *>(ws + L.order);
     b.item_off = reinterpret_cast<int64_t *>(ws + L.item_off);
     b.n_sys = n_sys;
-    b.pad = 0;
+    rc = batch_queues(&b.n_queues);
+    if (rc) return rc;
 
     EvalArgs a{};
     a.n_src = n_total;
