@@ -63,7 +63,9 @@ extern "C" {
 #define GRAV_FLAG_OVERFLOW  16 /* a tree build or walk exceeded its node bound (not expected) */
 
 /* Arithmetic of the force sums. */
-#define GRAV_F64   0  /* all pair arithmetic and sums in FP64 */
+#define GRAV_F64   0  /* FP64 results: pair terms in FP64, or (open boundaries) in two-part
+                         FP32 with the closest pairs and the final sums in FP64, with the
+                         error of the FP64 sums (csrc/grav_df.cuh) */
 #define GRAV_MIXED 1  /* FP64 positions offset to FP32 per source tile, FP32 pair
                          arithmetic, compensated FP32 tile sums, FP64 final sums */
 

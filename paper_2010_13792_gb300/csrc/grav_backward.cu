@@ -7,7 +7,8 @@
 // obtained by differentiating a_i = G sum_j m_j f(r) d (Eq. 4's acceleration)
 // with respect to x_k and m_k; T_k = d a_k / d x_k is the forward tidal tensor.
 // The paper has no adjoint.  The kernels are the forward direct sum with the
-// source attribute a_bar_i in place of (v_i, m_i) (FP64: backward_kernel;
+// source attribute a_bar_i in place of (v_i, m_i) (FP64: backward_kernel, pair
+// terms in two-part FP32 as in grav_df.cuh;
 // mixed: backward_pair_kernel on the forward's paired FP32x2 tile layout and
 // per-warp TMA ring): per pair they accumulate
 //   X1 += f a_bar_i,   X2 += g' (d . a_bar_i) d,   MB += f (d . a_bar_i)
@@ -43,64 +44,6 @@ struct BwdArgs {
     int32_t *flags;
     const float *src_lo;   // mixed: per tile, kLoPlanes planes (x, y, z) of the offsets' low parts
 };
-
-template <typename T>
-__device__ __forceinline__ T rsqrt_t(T x);
-template <>
-__device__ __forceinline__ double rsqrt_t<double>(double x) { return rsqrt(x); }
-
-template <typename T>
-__device__ __forceinline__ T sqrt_t(T x) { return sqrt(x); }
-
-template <typename T>
-struct Src;
-template <>
-struct Src<double> { using type = D4; };
-
-template <typename T, int KT, int S, bool NEAR>
-__device__ __forceinline__ void bwd_loop(const typename Src<T>::type *__restrict__ sp,
-                                         const typename Src<T>::type *__restrict__ sa,
-                                         const T tx[KT][3], const int64_t tk[KT], int64_t jbase,
-                                         T h2, T hinv, T acc[KT][kNB])
-{
-    const T hinv3 = hinv * hinv * hinv;
-    const T hinv5 = hinv3 * hinv * hinv;
-#pragma unroll 4
-    for (int j = 0; j < S; ++j) {
-        const auto p = sp[j];
-        const auto ab = sa[j];
-#pragma unroll
-        for (int q = 0; q < KT; ++q) {
-            // explicit fused multiply-adds: every kernel that inlines this
-            // loop forms the same roundings
-            T dx = p.x - tx[q][0], dy = p.y - tx[q][1], dz = p.z - tx[q][2];
-            T r2 = fma(dx, dx, fma(dy, dy, dz * dz));
-            T ri = rsqrt_t<T>(r2);
-            T ri2 = ri * ri;
-            T f = ri * ri2;
-            T gp = f * ri2;
-            if (NEAR && r2 < h2) {
-                T F, Gp, P;
-                spline_kernel<T>(sqrt_t<T>(r2) * hinv, F, Gp, P);
-                f = F * hinv3;
-                gp = Gp * hinv5;
-                if (jbase + j == tk[q]) {
-                    f = T(0);
-                    gp = T(0);
-                }
-            }
-            T da = fma(dx, ab.x, fma(dy, ab.y, dz * ab.z));
-            acc[q][X10 + 0] = fma(f, ab.x, acc[q][X10 + 0]);
-            acc[q][X10 + 1] = fma(f, ab.y, acc[q][X10 + 1]);
-            acc[q][X10 + 2] = fma(f, ab.z, acc[q][X10 + 2]);
-            T gd = gp * da;
-            acc[q][X20 + 0] = fma(gd, dx, acc[q][X20 + 0]);
-            acc[q][X20 + 1] = fma(gd, dy, acc[q][X20 + 1]);
-            acc[q][X20 + 2] = fma(gd, dz, acc[q][X20 + 2]);
-            acc[q][MBS] = fma(f, da, acc[q][MBS]);
-        }
-    }
-}
 
 __device__ __forceinline__ void bwd_write(const BwdArgs &a, int64_t k, const double s[kNB])
 {
@@ -139,203 +82,322 @@ struct BwdItem {
     int32_t t_begin, t_end, sp, split;
 };
 
-// Shared memory of the scalar adjoint: a two-stage ring of (x, a_bar) tiles.
-template <typename T, int S>
-struct BwdScalarSmem {
-    typename Src<T>::type stage[2][2 * S];
-    uint64_t bar[2];
-    float blo[3], bhi[3];
+// Shared memory of the FP64 adjoint: a two-stage ring of two-part (x, a_bar)
+// tiles, and the targets' running FP64 sums (hi, lo).
+template <int NT, int S>
+struct BwdDfSmem {
+    static constexpr int kStages = 2;
+    float stage[kStages][df_words<S>()];
+    double sum[kNB][2][NT];
+    uint64_t bar[kStages];
+    int done[kStages];           // warps finished with the tile in each stage
+    unsigned issued[kStages];    // copies issued into each stage
     int abort_flag;
     long long ticket;
 };
 
-template <typename Sm>
-__device__ __forceinline__ void bwd_init_ring(Sm &sm, int stages)
+// One sub-block of 32 sources of the FP64 adjoint in two-part arithmetic (the
+// forward's df_sub_loop with a_bar in the velocity's place and no mass).
+template <bool LIST, typename Add>
+__device__ __forceinline__ void bwd_df_loop(const float4 *__restrict__ P, const DfTarget &tg, float w3,
+                                            float w2, float thr2, DfSum (&sums)[kNB], Add &&list)
 {
-    if (threadIdx.x == 0) {
-        for (int s = 0; s < stages; ++s) mbar_init(&sm.bar[s], 1);
-        sm.abort_flag = 0;
-        fence_barrier_init();
-    }
-    __syncthreads();
-}
-
-// One item of the direct-sum adjoint on scalar (x, a_bar) tiles
-// (instantiated for FP64; the mixed adjoint is bwd_pair_item below); false
-// once a bounded wait gave up.  h2f_up: the FP32 squared support rounded up,
-// for the near-tile test.
-template <typename T, int NT, int KT, int S>
-__device__ __forceinline__ bool bwd_scalar_item(const BwdArgs &a, BwdScalarSmem<T, S> &sm,
-                                                uint32_t &parity, uint32_t &pending,
-                                                const BwdItem &it, T h2, T hinv, float h2f_up)
-{
-    using E = typename Src<T>::type;
-    constexpr bool MIXED = sizeof(T) == 4;
-    constexpr int NSTAGE = 2;
-    constexpr uint32_t kTileBytes = S * 2 * sizeof(E);
-    const E *src = static_cast<const E *>(a.src);
-    const int t_begin = it.t_begin, t_end = it.t_end;
-
-    double xk[KT][3];
-    int64_t tk[KT];
-    float lo[3], hi[3];
+    const float2 C3 = dup2(w3), C32 = dup2(df_second(w3)), C2 = dup2(w2), C22 = dup2(df_second(w2));
+#pragma unroll 1
+    for (int k0 = 0; k0 < kDfSub / 2; k0 += kDfCarry) {
+#pragma unroll 1
+        for (int k = k0; k < k0 + kDfCarry; ++k) {
+            const float4 *r = P + 7 * k;
+            const float4 q0 = r[0], q1 = r[1], q2 = r[2];
+            float2 d[3], e[3];
+            df_diff(make_float2(q0.x, q0.y), make_float2(q1.z, q1.w), -tg.h[0], -tg.l[0], -tg.l2[0], d[0],
+                    e[0]);
+            df_diff(make_float2(q0.z, q0.w), make_float2(q2.x, q2.y), -tg.h[1], -tg.l[1], -tg.l2[1], d[1],
+                    e[1]);
+            df_diff(make_float2(q1.x, q1.y), make_float2(q2.z, q2.w), -tg.h[2], -tg.l[2], -tg.l2[2], d[2],
+                    e[2]);
+            float2 r2h, r2l, sq;
+            df_square3(d, e, r2h, r2l, sq);
+            const float4 q3 = r[3], q4 = r[4], q5 = r[5];
+            float2 ah[3] = {make_float2(q3.x, q3.y), make_float2(q3.z, q3.w), make_float2(q4.x, q4.y)};
+            float2 al[3] = {make_float2(q4.z, q4.w), make_float2(q5.x, q5.y), make_float2(q5.z, q5.w)};
+            if (LIST && !(fminf(r2h.x, r2h.y) >= thr2)) {
+                // (listed, or padding: no a_bar at distance 1 instead)
+                if (!(r2h.x >= thr2)) {
+                    list(2 * k);
 #pragma unroll
-    for (int c = 0; c < 3; ++c) {
-        lo[c] = __int_as_float(0x7f800000);
-        hi[c] = -__int_as_float(0x7f800000);
-    }
+                    for (int c = 0; c < 3; ++c) ah[c].x = al[c].x = 0.0f;
+                    r2l.x = sq.x = 0.0f;
+                    r2h.x = 1.0f;
+                }
+                if (!(r2h.y >= thr2)) {
+                    list(2 * k + 1);
 #pragma unroll
-    for (int q = 0; q < KT; ++q) {
-        const int64_t k = it.k0 + (int64_t)q * NT + threadIdx.x;
-        tk[q] = k < it.k_end ? k : -1;
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            xk[q][c] = tk[q] >= 0 ? a.pos[3 * k + c] : 0.0;
-            if (tk[q] >= 0) {
-                lo[c] = fminf(lo[c], __double2float_rd(xk[q][c]));
-                hi[c] = fmaxf(hi[c], __double2float_ru(xk[q][c]));
+                    for (int c = 0; c < 3; ++c) ah[c].y = al[c].y = 0.0f;
+                    r2l.y = sq.y = 0.0f;
+                    r2h.y = 1.0f;
+                }
             }
-        }
-    }
-    block_bbox<NT>(lo, hi, sm.blo, sm.bhi);
-    // each warp tests tiles against its own targets' box (lo/hi now hold
-    // it): the near and far loops synchronise nothing
-    const float blo_r[3] = {lo[0], lo[1], lo[2]};
-    const float bhi_r[3] = {hi[0], hi[1], hi[2]};
-
-    T shi[KT][kNB], slo[KT][kNB];
-#pragma unroll
-    for (int q = 0; q < KT; ++q)
-#pragma unroll
-        for (int c = 0; c < kNB; ++c) {
-            shi[q][c] = T(0);
-            slo[q][c] = T(0);
-        }
-    if (threadIdx.x == 0) {
-        for (int s = 0; s < NSTAGE; ++s) {
-            int t = t_begin + s;
-            if (t < t_end) {
-                tma_load_1d(sm.stage[s], src + (int64_t)t * 2 * S, kTileBytes, &sm.bar[s]);
-                pending |= 1u << s;
-            }
-        }
-    }
-    for (int t = t_begin; t < t_end; ++t) {
-        const int s = (t - t_begin) % NSTAGE;
-        const TileGeom g = a.geo[t];
-        const bool near = tile_is_near(blo_r, bhi_r, g, h2f_up);
-        T tx[KT][3];
-#pragma unroll
-        for (int q = 0; q < KT; ++q)
+            const DfInv inv = df_inverse(r2h, r2l, sq);
+            float2 fh, fl, gh, gl, dah, dal, xh, xl;
+            df_inv3(inv, fh, fl);
+            df_times_inv2(inv, fh, fl, gh, gl);
+            df_dot3(d, e, ah, al, dah, dal);
+            df_mul(gh, gl, dah, dal, xh, xl);
 #pragma unroll
             for (int c = 0; c < 3; ++c) {
-                if (MIXED)
-                    tx[q][c] = (T)__double2float_rn(__dsub_rn(xk[q][c], g.c[c]));
-                else
-                    tx[q][c] = (T)xk[q][c];
+                df_add_product(sums[X10 + c], C3, C32, fh, fl, ah[c], al[c]);
+                df_add_product(sums[X20 + c], C3, C32, xh, xl, d[c], e[c]);
             }
-        const bool got = mbar_wait_bounded(&sm.bar[s], (parity >> s) & 1u, a.flags);
-        if (got)
-            parity ^= 1u << s;
-        else
-            atomicExch(&sm.abort_flag, 1);
-        T acc[KT][kNB];
+            df_add_product(sums[MBS], C2, C22, fh, fl, dah, dal);
+        }
 #pragma unroll
-        for (int q = 0; q < KT; ++q)
+        for (int c = 0; c < kNB; ++c) df_carry(sums[c], c == MBS ? C22 : C32);
+    }
+}
+
+// One pair of the adjoint in FP64 (d, a_bar given): added to s[kNB].  The
+// Newtonian powers are corrected for the rounding of rsqrt as in the forward.
+__device__ __forceinline__ void bwd_pair_fp64(const double d[3], const double ab[3], double h2, double hinv,
+                                              double hinv3, double hinv5, bool self, double s[kNB])
+{
+    const double r2 = fma(d[0], d[0], fma(d[1], d[1], d[2] * d[2]));
+    const double ri = rsqrt(r2);
+    const double ri2 = ri * ri;
+    const double t = fma(-r2, fma(ri, ri, -ri2), fma(-r2, ri2, 1.0));
+    double f = ri * ri2;
+    f = fma(f, 1.5 * t, f);
+    double gp = f * ri2;
+    gp = fma(gp, t, gp);
+    if (r2 < h2) {
+        double F, Gp, P;
+        spline_kernel<double>(sqrt(r2) * hinv, F, Gp, P);
+        f = F * hinv3;
+        gp = Gp * hinv5;
+        if (self) {
+            f = 0.0;
+            gp = 0.0;
+        }
+    }
+    const double da = fma(d[0], ab[0], fma(d[1], ab[1], d[2] * ab[2]));
+    const double gd = gp * da;
 #pragma unroll
-            for (int c = 0; c < kNB; ++c) acc[q][c] = T(0);
-        if (!near)
-            bwd_loop<T, KT, S, false>(sm.stage[s], sm.stage[s] + S, tx, tk, g.first, h2, hinv, acc);
-        else
-            bwd_loop<T, KT, S, true>(sm.stage[s], sm.stage[s] + S, tx, tk, g.first, h2, hinv, acc);
+    for (int c = 0; c < 3; ++c) {
+        s[X10 + c] = fma(f, ab[c], s[X10 + c]);
+        s[X20 + c] = fma(gd, d[c], s[X20 + c]);
+    }
+    s[MBS] = fma(f, da, s[MBS]);
+}
+
+__device__ __forceinline__ void bwd_add_sums(double *sum, int stride, const double acc[kNB])
+{
 #pragma unroll
-        for (int q = 0; q < KT; ++q)
+    for (int c = 0; c < kNB; ++c) {
+        double hi = sum[2 * c * stride], lo = sum[(2 * c + 1) * stride];
+        two_sum_ordered(hi, lo, acc[c]);
+        sum[2 * c * stride] = hi;
+        sum[(2 * c + 1) * stride] = lo;
+    }
+}
+
+// The listed pairs of target k, added to its running sums.
+__device__ __noinline__ void bwd_df_flush(const double *__restrict__ pos, const double *__restrict__ a_bar,
+                                          double h, int64_t k, const int32_t *list, int cnt, double *sum,
+                                          int stride)
+{
+    double acc[kNB];
 #pragma unroll
-            for (int c = 0; c < kNB; ++c) two_sum_ordered(shi[q][c], slo[q][c], acc[q][c]);
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            if (got) pending &= ~(1u << s);
-            if (t + NSTAGE < t_end && !sm.abort_flag) {
-                tma_load_1d(sm.stage[s], src + (int64_t)(t + NSTAGE) * 2 * S, kTileBytes, &sm.bar[s]);
-                pending |= 1u << s;
+    for (int c = 0; c < kNB; ++c) acc[c] = 0.0;
+    const double xk[3] = {pos[3 * k], pos[3 * k + 1], pos[3 * k + 2]};
+    const double h2 = h * h, hinv = 1.0 / h;
+    const double hinv3 = hinv * hinv * hinv, hinv5 = hinv3 * hinv * hinv;
+    for (int q = 0; q < cnt; ++q) {
+        const int64_t j = list[q];
+        const double d[3] = {pos[3 * j] - xk[0], pos[3 * j + 1] - xk[1], pos[3 * j + 2] - xk[2]};
+        const double ab[3] = {a_bar[3 * j], a_bar[3 * j + 1], a_bar[3 * j + 2]};
+        bwd_pair_fp64(d, ab, h2, hinv, hinv3, hinv5, false, acc);
+    }
+    bwd_add_sums(sum, stride, acc);
+}
+
+// One item of the FP64 adjoint (structure and reasons: df_item of the forward,
+// grav_eval_df.cuh); false once a bounded wait gave up.
+template <int NT, int S>
+__device__ __forceinline__ bool bwd_df_item(const BwdArgs &a, BwdDfSmem<NT, S> &sm, Ring &ring,
+                                            const BwdItem &it, double h)
+{
+    constexpr int NSTAGE = BwdDfSmem<NT, S>::kStages;
+    const char *src = static_cast<const char *>(a.src);
+    const int t_begin = it.t_begin, t_end = it.t_end;
+    const int64_t i = it.k0 + threadIdx.x;
+    const bool live = i < it.k_end;
+    double xk[3] = {0.0, 0.0, 0.0};
+    if (live) {
+#pragma unroll
+        for (int c = 0; c < 3; ++c) xk[c] = a.pos[3 * i + c];
+    }
+    double *sum = &sm.sum[0][0][threadIdx.x];
+#pragma unroll
+    for (int c = 0; c < 2 * kNB; ++c) sum[c * NT] = 0.0;
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < NSTAGE; ++s) {
+            const int t = t_begin + s;
+            if (t < t_end) {
+                tma_load_1d(sm.stage[s], src + t * df_stride<S>(), df_bytes<S>(), &sm.bar[s]);
+                sm.issued[s] += 1u;
             }
         }
-        if (sm.abort_flag) break;
     }
+    const bool warp_live = __any_sync(0xffffffffu, live);
+    int32_t list[kDfList];
+    int cnt = 0;
+    for (int t = t_begin; t < t_end; ++t) {
+        const int s = (t - t_begin) % NSTAGE;
+        const bool got = mbar_wait_bounded(&sm.bar[s], (ring.parity >> s) & 1u, a.flags);
+        if (got)
+            ring.parity ^= 1u << s;
+        else
+            atomicExch(&sm.abort_flag, 1);
+        if (warp_live && got) {
+            const TileGeom g = a.geo[t];
+            const float *tile = sm.stage[s];
+            const DfHead head = *reinterpret_cast<const DfHead *>(tile);
+            DfTarget tg;
+            const double il = df_offset(head, g.c, xk, tg);
+            const DfClass k = df_classify(tile, head, tg, live, h, il);
+            const int el = head.el, n_sub = (head.count + kDfSub - 1) / kDfSub;
+            double acc[kNB];
 #pragma unroll
-    for (int q = 0; q < KT; ++q) {
-        double sum[kNB];
+            for (int c = 0; c < kNB; ++c) acc[c] = 0.0;
+            const int n_df = n_sub - __popc(k.direct);
+            if (n_df > 0) {
+                DfSum sums[kNB];
 #pragma unroll
-        for (int c = 0; c < kNB; ++c) sum[c] = (double)shi[q][c] + (double)slo[q][c];
-        const int64_t slot = it.slot0 + (int64_t)q * NT + threadIdx.x;
+                for (int c = 0; c < kNB; ++c) sums[c] = DfSum{0u, 0u, make_float2(0.0f, 0.0f)};
+                const float i1 = rsqrt_sfu(k.rmin2) * (1.0f + 0x1p-18f);
+                // f a_bar, g (d.a_bar) d <= sqrt(3) r^-3; f (d.a_bar) <= sqrt(3) r^-2
+                const float w3 = df_window(1.8f * (i1 * i1 * i1)), w2 = df_window(1.8f * (i1 * i1));
+                const float4 *P = reinterpret_cast<const float4 *>(tile + df_records<S>());
+                for (int q = 0; q < n_sub; ++q) {
+                    if ((k.direct >> q) & 1u) continue;
+                    const float4 *Pq = P + 7 * (kDfSub / 2) * q;
+                    if ((k.close >> q) & 1u) {
+                        if (__any_sync(0xffffffffu, cnt > kDfList - kDfSub)) {
+                            if (cnt > 0) bwd_df_flush(a.pos, a.a_bar, h, i, list, cnt, sum, NT);
+                            cnt = 0;
+                            __syncwarp();
+                        }
+                        const int64_t j0 = g.first + kDfSub * q;
+                        const int real = min(kDfSub, head.count - kDfSub * q);
+                        auto add = [&](int j) {
+                            if (live && j < real && j0 + j != i) list[cnt++] = (int32_t)(j0 + j);
+                        };
+                        bwd_df_loop<true>(Pq, tg, w3, w2,
+                                          df_radius2(k, df_diagonal2(tile + kDfHeader + 6 * q)), sums, add);
+                    } else {
+                        bwd_df_loop<false>(Pq, tg, w3, w2, 0.0f, sums, [](int) {});
+                    }
+                }
+                const uint32_t n1 = kDfSub * n_df, n2 = n1 + n1 / kDfCarry;
+                const double u3 = pow2d(head.ev - 3 * el), u2 = pow2d(head.ev - 2 * el);
+#pragma unroll
+                for (int c = 0; c < kNB; ++c)
+                    acc[c] = df_value(sums[c], c == MBS ? w2 : w3, n1, n2, c == MBS ? u2 : u3);
+            }
+            if (k.direct) {
+                const double h2 = h * h, hinv = 1.0 / h;
+                const double hinv3 = hinv * hinv * hinv, hinv5 = hinv3 * hinv * hinv;
+                for (int q = 0; q < n_sub; ++q) {
+                    if (!((k.direct >> q) & 1u)) continue;
+                    const int real = min(kDfSub, head.count - kDfSub * q);
+                    for (int m = 0; m < real; ++m) {
+                        const int64_t j = g.first + kDfSub * q + m;
+                        const double d[3] = {a.pos[3 * j] - xk[0], a.pos[3 * j + 1] - xk[1],
+                                             a.pos[3 * j + 2] - xk[2]};
+                        const double ab[3] = {a.a_bar[3 * j], a.a_bar[3 * j + 1], a.a_bar[3 * j + 2]};
+                        bwd_pair_fp64(d, ab, h2, hinv, hinv3, hinv5, j == i, acc);
+                    }
+                }
+            }
+            bwd_add_sums(sum, NT, acc);
+        }
+        // this warp is done reading stage s; the last warp refills it
+        __syncwarp();
+        if ((threadIdx.x & 31) == 0) {
+            __threadfence_block();
+            const int prev = atomicAdd(&sm.done[s], 1);
+            if (prev == NT / 32 - 1) {
+                sm.done[s] = 0;
+                __threadfence_block();
+                if (t + NSTAGE < t_end && !*(volatile int *)&sm.abort_flag) {
+                    fence_proxy_async_smem();
+                    tma_load_1d(sm.stage[s], src + (t + NSTAGE) * df_stride<S>(), df_bytes<S>(), &sm.bar[s]);
+                    sm.issued[s] += 1u;
+                }
+            }
+        }
+        __syncwarp();
+        if (*(volatile int *)&sm.abort_flag) break;
+    }
+    __syncthreads();   // every warp is out of the tile loop: a uniform status
+    if (cnt > 0) bwd_df_flush(a.pos, a.a_bar, h, i, list, cnt, sum, NT);
+    if (live) {
+        double total[kNB];
+#pragma unroll
+        for (int c = 0; c < kNB; ++c) total[c] = __dadd_rn(sum[2 * c * NT], sum[(2 * c + 1) * NT]);
         if (it.split == 1) {
-            if (tk[q] >= 0) bwd_write(a, tk[q], sum);
+            bwd_write(a, i, total);
         } else {
+            const int64_t slot = it.slot0 + threadIdx.x;
 #pragma unroll
-            for (int c = 0; c < kNB; ++c) a.part[((int64_t)it.sp * kNB + c) * it.rows + slot] = sum[c];
+            for (int c = 0; c < kNB; ++c) a.part[((int64_t)it.sp * kNB + c) * it.rows + slot] = total[c];
         }
     }
     return !sm.abort_flag;
 }
 
-template <typename Sm>
-__device__ __forceinline__ void bwd_drain_scalar(Sm &sm, uint32_t parity, uint32_t pending,
-                                                 int32_t *flags)
-{
-    if (threadIdx.x == 0 && pending) {
-        for (int s = 0; s < 2; ++s)
-            if (pending & (1u << s)) mbar_wait_bounded(&sm.bar[s], (parity >> s) & 1u, flags);
-    }
-}
-
-// The scalar adjoint over all n elements: work items of target blocks x
-// source chunks.
-template <typename T, int NT, int KT, int S, int MINB>
+// The FP64 adjoint over all n elements: work items of target blocks x source
+// chunks.
+template <int NT, int S, int MINB>
 __global__ void __launch_bounds__(NT, MINB)
 backward_kernel(const BwdArgs a)
 {
-    constexpr bool MIXED = sizeof(T) == 4;
-    constexpr int BT = NT * KT;
-    __shared__ __align__(128) BwdScalarSmem<T, S> sm;
-    bwd_init_ring(sm, 2);
-    uint32_t parity = 0, pending = 0;
-
-    const int64_t n_tb = (a.n + BT - 1) / BT;
-    const int split = choose_split(n_tb, a.n_tiles, a.grid, a.max_split, a.part_cap_rows, BT);
+    extern __shared__ __align__(128) unsigned char smem_raw[];
+    auto &sm = *reinterpret_cast<BwdDfSmem<NT, S> *>(smem_raw);
+    init_mixed_ring(sm);
+    Ring ring{0u, 0u};
+    const int64_t n_tb = (a.n + NT - 1) / NT;
+    const int split = choose_split(n_tb, a.n_tiles, a.grid, a.max_split, a.part_cap_rows, NT);
     const int64_t items = n_tb * split;
-    const int64_t rows = n_tb * BT;
-    const T h2 = MIXED ? (T)a.h2f_up : (T)(a.h * a.h);
-    const T hinv = MIXED ? (T)a.hinvf : (T)(1.0 / a.h);
-
     for (int64_t item = blockIdx.x; item < items; item += gridDim.x) {
         const uint32_t tb = (uint32_t)item / (uint32_t)split;      // (32 bits, as the forward's)
         const int sp = (int)((uint32_t)item - tb * (uint32_t)split);
         BwdItem it;
-        it.k0 = (int64_t)tb * BT;
+        it.k0 = (int64_t)tb * NT;
         it.k_end = a.n;
-        it.slot0 = (int64_t)tb * BT;
-        it.rows = rows;
+        it.slot0 = (int64_t)tb * NT;
+        it.rows = n_tb * NT;
         it.t_begin = chunk_begin(sp, a.n_tiles, split);
         it.t_end = chunk_begin(sp + 1, a.n_tiles, split);
         it.sp = sp;
         it.split = split;
-        if (!bwd_scalar_item<T, NT, KT, S>(a, sm, parity, pending, it, h2, hinv, a.h2f_up)) break;
+        if (!bwd_df_item<NT, S>(a, sm, ring, it, a.h)) break;
         __syncthreads();
     }
-    bwd_drain_scalar(sm, parity, pending, a.flags);
+    drain_mixed_ring(sm, ring, a.flags);
 }
 
-// Batched scalar adjoint: the items of all systems from the plan, taken
-// from the per-SM queues; each system's targets against its own tiles
-// with its own support h (grav_system.h, or the call's h where it is 0).
-template <int NT, int KT, int S, int MINB>
+// Batched FP64 adjoint: the items of all systems from the plan, taken from
+// the per-SM queues; each system's targets against its own tiles with its own
+// support h (grav_system.h, or the call's h where it is 0).
+template <int NT, int S, int MINB>
 __global__ void __launch_bounds__(NT, MINB)
 backward_batched_kernel(const BwdArgs a, const BatchView b)
 {
-    constexpr int BT = NT * KT;
-    __shared__ __align__(128) BwdScalarSmem<double, S> sm;
-    bwd_init_ring(sm, 2);
-    uint32_t parity = 0, pending = 0;
+    extern __shared__ __align__(128) unsigned char smem_raw[];
+    auto &sm = *reinterpret_cast<BwdDfSmem<NT, S> *>(smem_raw);
+    init_mixed_ring(sm);
+    Ring ring{0u, 0u};
     const int64_t total = b.hdr->total_items;
     for (;;) {
         if (threadIdx.x < 32) {
@@ -349,10 +411,8 @@ backward_batched_kernel(const BwdArgs a, const BatchView b)
         const int r = item_rank(b, ticket);
         const int s = b.order[r];
         const double h = b.sys[s].h > 0.0 ? b.sys[s].h : a.h;
-        float h2f, hinvf;
-        softening_f(h, h2f, hinvf);
         BwdItem it;
-        it.k0 = (int64_t)b.idx_lo[s] + (ticket - b.item_off[r]) * BT;
+        it.k0 = (int64_t)b.idx_lo[s] + (ticket - b.item_off[r]) * NT;
         it.k_end = b.idx_hi[s];
         it.slot0 = 0;
         it.rows = 0;
@@ -360,10 +420,10 @@ backward_batched_kernel(const BwdArgs a, const BatchView b)
         it.t_end = b.tile_off[s + 1];
         it.sp = 0;
         it.split = 1;
-        if (!bwd_scalar_item<double, NT, KT, S>(a, sm, parity, pending, it, h * h, 1.0 / h, h2f)) break;
+        if (!bwd_df_item<NT, S>(a, sm, ring, it, h)) break;
         __syncthreads();
     }
-    bwd_drain_scalar(sm, parity, pending, a.flags);
+    drain_mixed_ring(sm, ring, a.flags);
 }
 
 // Mixed adjoint on the paired source layout of the forward kernel (the
@@ -848,12 +908,21 @@ __global__ void __launch_bounds__(256) backward_pot_only_kernel(const BwdArgs a)
 // Fixed tile shapes of the adjoint.
 constexpr int kBwdNTf = 768, kBwdKTf = 1, kBwdSf = 256, kBwdMinBf = 1, kBwdUf = 4;
 constexpr size_t kBwdSmemf = sizeof(BwdPairSmem<kBwdSf>);
-constexpr int kBwdNTd = 128, kBwdKTd = 1, kBwdSd = 128, kBwdMinBd = 2;
+// FP64: 256-source tiles, 128 below 2^25 pairs (as the forward: kFinePairs)
+constexpr int kBwdNTd = 128, kBwdSd = 256, kBwdSfine = 128, kBwdMinBd = 4;
+constexpr int64_t kBwdFinePairs = 1LL << 25;
+constexpr size_t kBwdSmemd = sizeof(BwdDfSmem<kBwdNTd, kBwdSd>);
+constexpr size_t kBwdSmemfine = sizeof(BwdDfSmem<kBwdNTd, kBwdSfine>);
 
 struct BwdLayout {
     int64_t n_tiles, geo_off, src_off, lo_off, part_off, total, part_cap_rows;
     int32_t max_split, S, BT;
 };
+
+bool bwd_fine(const grav_params *p, int64_t n)
+{
+    return p->precision == GRAV_F64 && p->max_split != 1 && n * n < kBwdFinePairs;
+}
 
 int bwd_layout(const grav_params *p, int64_t n, BwdLayout *L)
 {
@@ -861,14 +930,14 @@ int bwd_layout(const grav_params *p, int64_t n, BwdLayout *L)
     int rc = device_sm_count(&sms);
     if (rc) return rc;
     const bool mixed = p->precision == GRAV_MIXED;
-    L->S = mixed ? kBwdSf : kBwdSd;
-    L->BT = mixed ? kBwdNTf * kBwdKTf : kBwdNTd * kBwdKTd;
-    const int64_t elem = mixed ? 16 : 32;
+    L->S = mixed ? kBwdSf : bwd_fine(p, n) ? kBwdSfine : kBwdSd;
+    L->BT = mixed ? kBwdNTf * kBwdKTf : kBwdNTd;
+    const int64_t bytes = mixed ? 32 : kDfBytesPerSource;
     L->max_split = p->max_split > 0 ? p->max_split : kDefaultMaxSplit;
     L->n_tiles = (n + L->S - 1) / L->S;
     L->geo_off = 0;
     L->src_off = round_up(L->n_tiles * (int64_t)sizeof(TileGeom), 256);
-    L->lo_off = L->src_off + round_up(L->n_tiles * 2 * L->S * elem, 256);
+    L->lo_off = L->src_off + round_up(L->n_tiles * L->S * bytes, 256);
     L->part_off = L->lo_off + round_up(mixed ? L->n_tiles * kLoPlanes * L->S * 4 : 0, 256);
     const int64_t n_tb = (n + L->BT - 1) / L->BT;
     int64_t blocks = 0;
@@ -878,10 +947,10 @@ int bwd_layout(const grav_params *p, int64_t n, BwdLayout *L)
     return GRAV_OK;
 }
 
-int bwd_grid(bool mixed, bool batched, int *grid)
+int bwd_grid(bool mixed, bool batched, bool fine, int *grid)
 {
     static std::mutex mu;
-    static int cache[64][2][2];
+    static int cache[64][2][3];
     int dev = 0, sms = 0;
     int rc = check_cuda(cudaGetDevice(&dev), "cudaGetDevice");
     if (rc) return rc;
@@ -889,7 +958,7 @@ int bwd_grid(bool mixed, bool batched, int *grid)
     if (rc) return rc;
     if (dev >= 64) return fail(GRAV_ECUDA, "device ordinal out of range");
     std::lock_guard<std::mutex> lk(mu);
-    int &slot = cache[dev][mixed ? 1 : 0][batched ? 1 : 0];
+    int &slot = cache[dev][mixed ? 1 : 0][batched ? 1 : fine ? 2 : 0];
     if (slot == 0) {
         int b = 0;
         cudaError_t e = cudaSuccess;
@@ -901,12 +970,17 @@ int bwd_grid(bool mixed, bool batched, int *grid)
             auto k = backward_pair_batched_kernel<kBwdNTf, kBwdKTf, kBwdSf, kBwdMinBf, kBwdUf>;
             e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBwdSmemf);
             if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k, kBwdNTf, kBwdSmemf);
-        } else if (!batched) {
-            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-                &b, backward_kernel<double, kBwdNTd, kBwdKTd, kBwdSd, kBwdMinBd>, kBwdNTd, 0);
         } else {
-            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-                &b, backward_batched_kernel<kBwdNTd, kBwdKTd, kBwdSd, kBwdMinBd>, kBwdNTd, 0);
+            auto set = [&](auto k, size_t bytes) {
+                e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+                if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k, kBwdNTd, bytes);
+            };
+            if (batched)
+                set(backward_batched_kernel<kBwdNTd, kBwdSd, kBwdMinBd>, kBwdSmemd);
+            else if (fine)
+                set(backward_kernel<kBwdNTd, kBwdSfine, kBwdMinBd>, kBwdSmemfine);
+            else
+                set(backward_kernel<kBwdNTd, kBwdSd, kBwdMinBd>, kBwdSmemd);
         }
         rc = check_cuda(e, "cudaOccupancyMaxActiveBlocksPerMultiprocessor");
         if (rc) return rc;
@@ -926,7 +1000,7 @@ BwdBatchLayout bwd_batch_layout(bool mixed, int32_t n_sys, int64_t n_total)
 {
     BwdBatchLayout L;
     const int64_t S = mixed ? kBwdSf : kBwdSd;
-    const int64_t elem = mixed ? 16 : 32;
+    const int64_t bytes = mixed ? 32 : kDfBytesPerSource;
     L.max_tiles = (n_total + S - 1) / S + n_sys;
     int64_t o = 0;
     L.hdr = o;
@@ -946,7 +1020,7 @@ BwdBatchLayout bwd_batch_layout(bool mixed, int32_t n_sys, int64_t n_total)
     L.geo = o;
     o += round_up(L.max_tiles * (int64_t)sizeof(TileGeom), 256);
     L.src = o;
-    o += round_up(L.max_tiles * 2 * S * elem, 256);
+    o += round_up(L.max_tiles * S * bytes, 256);
     L.lo = o;
     o += round_up(mixed ? L.max_tiles * kLoPlanes * S * 4 : 0, 256);
     L.total = o;
@@ -1008,7 +1082,8 @@ extern "C" int grav_eval_backward(const grav_params *p, int64_t n, const double 
                         (long long)L.total);
     }
     int grid = 0;
-    rc = bwd_grid(mixed, false, &grid);
+    const bool fine = bwd_fine(p, n);
+    rc = bwd_grid(mixed, false, fine, &grid);
     if (rc) return rc;
     char *ws = static_cast<char *>(workspace);
     BwdArgs a;
@@ -1051,15 +1126,20 @@ extern "C" int grav_eval_backward(const grav_params *p, int64_t n, const double 
         pack_tiles_kernel<kBwdSf, true, false, true><<<(unsigned)L.n_tiles, kBwdSf, 0, st>>>(
             n, pos, a_bar, nullptr, const_cast<TileGeom *>(a.geo), const_cast<void *>(a.src), flags_dev,
             const_cast<float *>(a.src_lo));
+    else if (fine)
+        pack_tiles_kernel<kBwdSfine, false, false, false, true><<<(unsigned)L.n_tiles, kBwdSfine, 0, st>>>(
+            n, pos, a_bar, nullptr, const_cast<TileGeom *>(a.geo), const_cast<void *>(a.src), flags_dev);
     else
-        pack_tiles_kernel<kBwdSd, false, false><<<(unsigned)L.n_tiles, kBwdSd, 0, st>>>(
+        pack_tiles_kernel<kBwdSd, false, false, false, true><<<(unsigned)L.n_tiles, kBwdSd, 0, st>>>(
             n, pos, a_bar, nullptr, const_cast<TileGeom *>(a.geo), const_cast<void *>(a.src), flags_dev);
     rc = check_launch("grav_eval_backward/pack");
     if (rc) return rc;
     if (mixed)
         backward_pair_kernel<kBwdNTf, kBwdKTf, kBwdSf, kBwdMinBf, kBwdUf><<<grid, kBwdNTf, kBwdSmemf, st>>>(a);
+    else if (fine)
+        backward_kernel<kBwdNTd, kBwdSfine, kBwdMinBd><<<grid, kBwdNTd, kBwdSmemfine, st>>>(a);
     else
-        backward_kernel<double, kBwdNTd, kBwdKTd, kBwdSd, kBwdMinBd><<<grid, kBwdNTd, 0, st>>>(a);
+        backward_kernel<kBwdNTd, kBwdSd, kBwdMinBd><<<grid, kBwdNTd, kBwdSmemd, st>>>(a);
     rc = check_launch("grav_eval_backward/sum");
     if (rc) return rc;
     const int64_t n_tb = (n + L.BT - 1) / L.BT;
@@ -1111,7 +1191,7 @@ extern "C" int grav_eval_backward_batched(const grav_params *p, int32_t n_sys,
         return fail(GRAV_ENOMEM, "%s: workspace of %lld bytes < %lld", who, (long long)workspace_bytes,
                     (long long)L.total);
     int grid = 0;
-    rc = bwd_grid(mixed, true, &grid);
+    rc = bwd_grid(mixed, true, false, &grid);
     if (rc) return rc;
     char *ws = static_cast<char *>(workspace);
     BatchView b;
@@ -1162,7 +1242,7 @@ extern "C" int grav_eval_backward_batched(const grav_params *p, int32_t n_sys,
         return check_launch("grav_eval_backward_batched/pot");
     }
     const int32_t S = mixed ? kBwdSf : kBwdSd;
-    const int32_t BT = mixed ? kBwdNTf * kBwdKTf : kBwdNTd * kBwdKTd;
+    const int32_t BT = mixed ? kBwdNTf * kBwdKTf : kBwdNTd;
     // every element a target: the plan takes each system's element range
     rc = launch_batch_plan(b, nullptr, nullptr, n_total, n_total, S, BT, 0.0, flags_dev, st);
     if (rc) return rc;
@@ -1173,7 +1253,7 @@ extern "C" int grav_eval_backward_batched(const grav_params *p, int32_t n_sys,
             b, pos, a_bar, nullptr, const_cast<TileGeom *>(a.geo), const_cast<void *>(a.src), flags_dev,
             const_cast<float *>(a.src_lo));
     else
-        pack_tiles_batched_kernel<kBwdSd, false, false, false><<<(unsigned)L.max_tiles, kBwdSd, 0, st>>>(
+        pack_tiles_batched_kernel<kBwdSd, false, false, false, true><<<(unsigned)L.max_tiles, kBwdSd, 0, st>>>(
             b, pos, a_bar, nullptr, const_cast<TileGeom *>(a.geo), const_cast<void *>(a.src), flags_dev,
             nullptr);
     rc = check_launch("grav_eval_backward_batched/pack");
@@ -1182,6 +1262,6 @@ extern "C" int grav_eval_backward_batched(const grav_params *p, int32_t n_sys,
         backward_pair_batched_kernel<kBwdNTf, kBwdKTf, kBwdSf, kBwdMinBf, kBwdUf>
             <<<grid, kBwdNTf, kBwdSmemf, st>>>(a, b);
     else
-        backward_batched_kernel<kBwdNTd, kBwdKTd, kBwdSd, kBwdMinBd><<<grid, kBwdNTd, 0, st>>>(a, b);
+        backward_batched_kernel<kBwdNTd, kBwdSd, kBwdMinBd><<<grid, kBwdNTd, kBwdSmemd, st>>>(a, b);
     return check_launch("grav_eval_backward_batched/sum");
 }

@@ -1,0 +1,453 @@
+// FP64-accurate pair sums in two-part FP32 arithmetic ("double-float").
+//
+// GB300 runs FP64 at 1/64 of its FP32 rate (2 FMA per clock and SM), and the
+// FP64 force kernel needs 39 FP64 instructions a pair: 2500 FP32 lane slots.
+// The same pair carried as unevaluated sums of two FP32 numbers (about 48 bits)
+// takes some 190 FP32 operations, two sources to a packed FP32x2 instruction.
+//
+// Pieces:
+//   * Tiles hold the sources' offsets from the tile centre in units of a power
+//     of two L, velocities in units V and masses in units of the largest mass
+//     M, so the FP32 range does not limit the caller's units and the rounding
+//     of a mass that all sources share does not bias the sums (it would be the
+//     same 2^-49 for each): x = sh + sl, each rounded to nearest.
+//   * Separations: Knuth's TwoSum of the high parts plus the difference of the
+//     low parts, renormalised.
+//   * r^-3 and r^-5 from y, the SFU's rsqrt after one FP32 Newton step: with
+//     t = 1 - r^2 y^2 formed from both parts, r^-3 = y^3 (1 + 3/2 t + 15/8 t^2),
+//     r^-2 = y^2 (1 + t + t^2) (the binomial series; |t| <= 2^-22, so the next
+//     terms are below 2^-64).
+//   * Sums: a product's high part p is split at the unit of a constant C =
+//     1.5 * 2^k that exceeds every |p|: p + C holds p rounded to a multiple of
+//     ulp(C) in its low mantissa bits, which are added up exactly as integers
+//     (one three-input integer add for two sources); the rest, exact, is cut
+//     a second time at the unit of a smaller constant, and what then remains
+//     joins the product's low part in an FP32 sum.  Nothing but that last sum
+//     is rounded, and it is 2^20 and more below the total even where the window
+//     is a thousand times wider than the sum (unequal masses).
+// A pair comes out good to about 8e-15 (rms, its force), and thousands of them
+// average; the pairs closest to a target, whose rounding would not, are listed
+// and summed in FP64.
+#pragma once
+
+#include "grav_common.cuh"
+
+namespace grav {
+
+// Words of a packed tile of S sources: an 8-word header, the boxes of its
+// sub-blocks of 32 sources (lo, hi in units of L, rounded outward), S/2
+// records of 28 floats (two sources side by side: xh yh zh xl yl zl, the same
+// of the velocity, mh ml).
+constexpr int kDfSub = 32;
+constexpr int kDfHeader = 8;
+template <int S>
+constexpr int df_records() { return kDfHeader + 6 * (S / kDfSub); }
+template <int S>
+constexpr int df_words() { return df_records<S>() + 14 * S; }
+template <int S>
+constexpr uint32_t df_bytes() { return 4u * df_words<S>(); }
+// stride of the tiles in the workspace
+constexpr int64_t kDfBytesPerSource = 58;
+template <int S>
+constexpr int64_t df_stride() { return kDfBytesPerSource * S; }
+static_assert(df_bytes<64>() <= df_stride<64>() && df_bytes<128>() <= df_stride<128>() &&
+              df_bytes<256>() <= df_stride<256>() && df_stride<64>() % 16 == 0, "DF tile stride");
+
+struct DfHead {
+    double munit;      // M: the largest |m| (1 if all are 0)
+    float ext[3];      // half extents / L, rounded up
+    int16_t el, ev;    // units: L = 2^el >= half extent, V = 2^ev > |v'|
+    int16_t ok;        // 0: out of the ranges above, the tile is summed in FP64
+    int16_t count;     // sources in the tile
+    int32_t pad;
+};
+static_assert(sizeof(DfHead) == 4 * kDfHeader, "DfHead layout");
+
+// A power of two above |x| of the largest high word hi (of |x|).
+__device__ __forceinline__ int exponent_above(uint32_t hi) { return (int)(hi >> 20) - 1022; }
+
+__device__ __forceinline__ double pow2d(int e)   // -1022 <= e <= 1023
+{
+    return __hiloint2double((e + 1023) << 20, 0);
+}
+
+__device__ __forceinline__ float2 dup2(float a) { return make_float2(a, a); }
+__device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
+// a - b, rounded once
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, dup2(-1.0f), a); }
+
+// Packs one tile (one CTA of S threads, thread j its source): `x` the FP64
+// offset from the tile centre, `v` the velocity relative to the tile's
+// velocity centre (or the adjoint's a_bar), m the mass; `half` the tile's half
+// extents.  Padding sources (!ok) copy the place of their sub-block's first
+// source with zero mass.  A warp is a sub-block.
+template <int S>
+__device__ __forceinline__ void df_pack(void *tile, int j, bool ok, int count, const double x[3],
+                                        const double v[3], double m, const double half[3], double cmax)
+{
+    __shared__ uint32_t wmax[3][S / 32];
+    const int lane = j & 31, wid = j >> 5;
+    uint32_t hv = 0, hm = 0, lm = 0;
+    if (ok) {
+#pragma unroll
+        for (int c = 0; c < 3; ++c) hv = max(hv, (uint32_t)__double2hiint(v[c]) & 0x7fffffffu);
+        hm = (uint32_t)__double2hiint(m) & 0x7fffffffu;
+        lm = (uint32_t)__double2loint(m);
+    }
+    hv = __reduce_max_sync(0xffffffffu, hv);
+    const uint32_t top = __reduce_max_sync(0xffffffffu, hm);
+    lm = __reduce_max_sync(0xffffffffu, hm == top ? lm : 0u);
+    hm = top;
+    if (lane == 0) {
+        wmax[0][wid] = hv;
+        wmax[1][wid] = hm;
+        wmax[2][wid] = lm;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int w = 0; w < S / 32; ++w) {
+        hv = max(hv, wmax[0][w]);
+        const uint32_t h2 = wmax[1][w], l2 = wmax[2][w];
+        lm = h2 > hm ? l2 : h2 == hm ? max(lm, l2) : lm;
+        hm = max(hm, h2);
+    }
+    uint32_t hx = 0;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) hx = max(hx, (uint32_t)__double2hiint(half[c]) & 0x7fffffffu);
+    // L no smaller than 2^-10 of the centre's distance from the origin: targets
+    // of a tile of coincident elements stay in range
+    const uint32_t hc = (uint32_t)__double2hiint(cmax) & 0x7fffffffu;
+    DfHead h;
+    int el = max(exponent_above(hx), exponent_above(hc) - 10);
+    if (hx == 0 && hc == 0) el = 0;
+    const int ev = hv == 0 ? 0 : exponent_above(hv);
+    const int em = hm == 0 ? 0 : exponent_above(hm);
+    h.ok = hx < 0x7ff00000u && hv < 0x7ff00000u && hm < 0x7ff00000u && abs(el) <= 150 &&
+           abs(ev) <= 150 && abs(em) <= 150;
+    el = max(-150, min(150, el));
+    h.el = (int16_t)el;
+    h.ev = (int16_t)max(-150, min(150, ev));
+    h.munit = h.ok && hm != 0 ? __hiloint2double((int)hm, (int)lm) : 1.0;
+    h.count = (int16_t)count;
+    h.pad = 0;
+    const double il = pow2d(-el);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) h.ext[c] = __double2float_ru(__dmul_rn(half[c], il));
+    float *out = static_cast<float *>(tile);
+    if (j == 0) *reinterpret_cast<DfHead *>(out) = h;
+    const double iv = pow2d(-h.ev);
+    float *rec = out + df_records<S>() + 28 * (j >> 1) + (j & 1);
+    float *box = out + kDfHeader + 6 * wid;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        const double s = __shfl_sync(0xffffffffu, __dmul_rn(x[c], il), ok ? lane : 0);
+        const float sh = __double2float_rn(s);
+        rec[2 * c] = sh;
+        rec[6 + 2 * c] = __double2float_rn(__dsub_rn(s, (double)sh));
+        float lo = __double2float_rd(s), hi = __double2float_ru(s);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+            hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+        }
+        if (lane == 0) {
+            box[c] = lo;
+            box[3 + c] = hi;
+        }
+        const double u = ok ? __dmul_rn(v[c], iv) : 0.0;
+        const float vh = __double2float_rn(u);
+        rec[12 + 2 * c] = vh;
+        rec[18 + 2 * c] = __double2float_rn(__dsub_rn(u, (double)vh));
+    }
+    const double w = ok ? __ddiv_rn(m, h.munit) : 0.0;
+    const float mh = __double2float_rn(w);
+    rec[24] = mh;
+    rec[26] = __double2float_rn(__dsub_rn(w, (double)mh));
+}
+
+// A target against one tile: offset from the tile centre in units of L, in
+// three parts (a pair's separation needs two; the third keeps the offset's own
+// rounding, which all pairs of the tile share, out of the sums).
+struct DfTarget {
+    float h[3], l[3], l2[3];
+};
+
+__device__ __forceinline__ void df_split(const double x[3], DfTarget &t)
+{
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        t.h[c] = __double2float_rn(x[c]);
+        const double r1 = __dsub_rn(x[c], (double)t.h[c]);
+        t.l[c] = __double2float_rn(r1);
+        t.l2[c] = __double2float_rn(__dsub_rn(r1, (double)t.l[c]));
+    }
+}
+
+// C = 1.5 * 2^k with 2^(k-1) > b (b > 0, normal).
+__device__ __forceinline__ float df_window(float b)
+{
+    return __uint_as_float((__float_as_uint(b) & 0x7f800000u) + (2u << 23) + 0x400000u);
+}
+
+// One two-part sum of a target over a tile: i1 counts units ulp(C), i2 units
+// ulp(C2), lo the rest (its two lanes the even and the odd sources).
+struct DfSum {
+    uint32_t i1, i2;
+    float2 lo;
+};
+
+// Second window of a sum: 2^4 units of C, so |rest| may reach 8 units.
+__device__ __forceinline__ float df_second(float C) { return __uint_as_float(__float_as_uint(C) - (19u << 23)); }
+
+// Moves the part of `lo` above ulp(C2) into the second integer sum.
+__device__ __forceinline__ void df_carry(DfSum &s, float2 C2)
+{
+    const float2 t = __fadd2_rn(s.lo, C2);
+    s.i2 += __float_as_uint(t.x) + __float_as_uint(t.y);
+    s.lo = __fadd2_rn(s.lo, sub2(C2, t));
+}
+
+// sum += (fh + fl) (dh + dl) for two sources; df_carry follows every
+// kDfCarry records.
+constexpr int kDfCarry = 8;
+
+__device__ __forceinline__ void df_add_product(DfSum &s, float2 C, float2 C2, float2 fh, float2 fl,
+                                               float2 dh, float2 dl)
+{
+    const float2 p = __fmul2_rn(fh, dh);
+    float2 w = __ffma2_rn(fh, dh, neg2(p));
+    w = __ffma2_rn(fh, dl, w);
+    w = __ffma2_rn(fl, dh, w);
+    const float2 t = __fadd2_rn(p, C);
+    s.i1 += __float_as_uint(t.x) + __float_as_uint(t.y);
+    const float2 r = __fadd2_rn(p, sub2(C, t));
+    const float2 u = __fadd2_rn(r, C2);
+    s.i2 += __float_as_uint(u.x) + __float_as_uint(u.y);
+    s.lo = __fadd2_rn(s.lo, __fadd2_rn(__fadd2_rn(r, sub2(C2, u)), w));
+}
+
+// The sum as FP64 in the caller's units (`unit` of the tile's), after n1
+// additions to i1 and n2 to i2.
+__device__ __forceinline__ double df_value(const DfSum &s, float C, uint32_t n1, uint32_t n2, double unit)
+{
+    const int a = (int)(s.i1 - n1 * __float_as_uint(C));
+    const int b = (int)(s.i2 - n2 * __float_as_uint(df_second(C)));
+    const long long n = ((long long)a << 19) + b;
+    const int e2 = (int)(__float_as_uint(C) >> 23) - 127 - 42;          // ulp(C2) = 2^e2
+    // (`unit` is normal and far from the ends: its exponent can be moved)
+    const double scale = __hiloint2double(__double2hiint(unit) + (e2 << 20), __double2loint(unit));
+    return __fma_rn((double)n, scale, __dmul_rn((double)__fadd_rn(s.lo.x, s.lo.y), unit));
+}
+
+// (ah + al) (bh + bl), high and low parts not renormalised.
+__device__ __forceinline__ void df_mul(float2 ah, float2 al, float2 bh, float2 bl, float2 &ph, float2 &pl)
+{
+    ph = __fmul2_rn(ah, bh);
+    pl = __ffma2_rn(ah, bh, neg2(ph));
+    pl = __ffma2_rn(ah, bl, pl);
+    pl = __ffma2_rn(al, bh, pl);
+}
+
+__device__ __forceinline__ void two_sum2(float2 a, float2 b, float2 &s, float2 &e)
+{
+    s = __fadd2_rn(a, b);
+    const float2 z = sub2(s, a);
+    e = __fadd2_rn(sub2(a, sub2(s, z)), sub2(b, z));
+}
+
+// h + l renormalised (|h| >= |l|): |l| at most half a unit of h.
+__device__ __forceinline__ void df_norm(float2 &h, float2 &l)
+{
+    const float2 s = __fadd2_rn(h, l);
+    l = sub2(l, sub2(s, h));
+    h = s;
+}
+
+// Separation component: source (sh, sl) minus target (n*: its parts negated).
+__device__ __forceinline__ void df_diff(float2 sh, float2 sl, float nh, float nl, float n2, float2 &d,
+                                        float2 &e)
+{
+    two_sum2(sh, dup2(nh), d, e);
+    e = __fadd2_rn(e, __fadd2_rn(sl, dup2(nl)));
+    df_norm(d, e);
+    e = __fadd2_rn(e, dup2(n2));
+}
+
+// Sum of three products (high parts TwoSum'd, not renormalised).
+__device__ __forceinline__ void df_dot3(const float2 ah[3], const float2 al[3], const float2 bh[3],
+                                        const float2 bl[3], float2 &ph, float2 &pl)
+{
+    float2 h[3], l[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) df_mul(ah[c], al[c], bh[c], bl[c], h[c], l[c]);
+    float2 s, e1, e2;
+    two_sum2(h[0], h[1], s, e1);
+    two_sum2(s, h[2], ph, e2);
+    pl = __fadd2_rn(__fadd2_rn(__fadd2_rn(l[0], l[1]), l[2]), __fadd2_rn(e1, e2));
+}
+
+// r^2, renormalised, without the squares of the low parts: those lie below
+// the last place of the result.  Being of one sign they would not average over
+// the pairs; their sum (sq) goes into the series instead (DfInv::s).
+__device__ __forceinline__ void df_square3(const float2 d[3], const float2 e[3], float2 &ph, float2 &pl,
+                                           float2 &sq)
+{
+    float2 h[3], l[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        h[c] = __fmul2_rn(d[c], d[c]);
+        l[c] = __ffma2_rn(__fadd2_rn(d[c], d[c]), e[c], __ffma2_rn(d[c], d[c], neg2(h[c])));
+    }
+    sq = __ffma2_rn(e[0], e[0], __ffma2_rn(e[1], e[1], __fmul2_rn(e[2], e[2])));
+    float2 s, e1, e2;
+    two_sum2(h[0], h[1], s, e1);
+    two_sum2(s, h[2], ph, e2);
+    pl = __fadd2_rn(__fadd2_rn(__fadd2_rn(l[0], l[1]), l[2]), __fadd2_rn(e1, e2));
+    df_norm(ph, pl);
+}
+
+// y = r^-1, t = 1 - r^2 y^2, y^2 as two parts, and s = -sq y^2, the part of t
+// below its last place (it is added to a product inside an fma, whose own
+// low bits keep it from being rounded away).
+struct DfInv {
+    float2 y, t, y2h, y2l, s;
+};
+
+__device__ __forceinline__ DfInv df_inverse(float2 r2h, float2 r2l, float2 sq)
+{
+    DfInv v;
+    const float2 n = neg2(r2h);
+    const float2 y0 = make_float2(rsqrt_sfu(r2h.x), rsqrt_sfu(r2h.y));
+    v.y = __ffma2_rn(__fmul2_rn(dup2(0.5f), y0), __ffma2_rn(__fmul2_rn(n, y0), y0, dup2(1.0f)), y0);
+    v.y2h = __fmul2_rn(v.y, v.y);
+    v.y2l = __ffma2_rn(v.y, v.y, neg2(v.y2h));
+    float2 t = __ffma2_rn(n, v.y2h, dup2(1.0f));
+    t = __ffma2_rn(n, v.y2l, t);
+    v.t = __ffma2_rn(neg2(r2l), v.y2h, t);
+    v.s = __fmul2_rn(neg2(sq), v.y2h);
+    return v;
+}
+
+// r^-3 (two parts).
+__device__ __forceinline__ void df_inv3(const DfInv &v, float2 &h, float2 &l)
+{
+    const float2 c = __ffma2_rn(v.t, __ffma2_rn(dup2(1.875f), v.t, dup2(1.5f)), __fmul2_rn(dup2(1.5f), v.s));
+    h = __fmul2_rn(v.y2h, v.y);
+    l = __ffma2_rn(v.y2h, v.y, neg2(h));
+    l = __ffma2_rn(v.y2l, v.y, l);
+    l = __ffma2_rn(h, c, l);
+    df_norm(h, l);
+}
+
+// Times r^-2.
+__device__ __forceinline__ void df_times_inv2(const DfInv &v, float2 fh, float2 fl, float2 &gh, float2 &gl)
+{
+    float2 h = v.y2h, l = __ffma2_rn(v.y2h, __ffma2_rn(v.t, v.t, v.t), v.y2l);
+    df_norm(h, l);
+    df_mul(fh, fl, h, l, gh, gl);
+}
+
+// Windows of one target against one tile (units of L, V, M): every term of an
+// accumulated sum stays below half its window's power of two.
+struct DfWindows {
+    float a, t, j, p;
+};
+
+// rmin2 <= r^2 of every pair that is summed.
+__device__ __forceinline__ DfWindows df_windows(float rmin2)
+{
+    DfWindows w;
+    const float i1 = rsqrt_sfu(rmin2) * (1.0f + 0x1p-18f);
+    const float i2 = i1 * i1;
+    w.a = df_window(i2);                 // m f d     <= r^-2
+    w.t = df_window(i2 * i1);            // m g d d   <= r^-3
+    w.j = df_window(1.8f * (i2 * i1));   // m f v <= r^-3, m g (d.v) d <= sqrt(3) r^-3 (|v_c| <= 1)
+    w.p = df_window(i1);                 // m phi     <= r^-1
+    return w;
+}
+
+// Where a tile's sub-blocks lie for the targets of a warp (one per lane).
+constexpr float kDfRange = 32768.0f;   // targets beyond this many L from a tile: FP64
+// Pairs closer than this share of the sub-block's diagonal (2.3 spacings of
+// its sources) are listed for FP64, and so are softened pairs.
+constexpr float kDfNear = 0.42f;
+constexpr int kDfList = 64;            // room for two sub-blocks per target
+
+struct DfClass {
+    uint32_t direct;   // sub-blocks summed in FP64 (softening wider than half their diagonal)
+    uint32_t close;    // sub-blocks with listed pairs
+    float rmin2;       // least r^2 of the pairs left to this lane's target
+    float floor2;      // least listing radius (squared)
+};
+
+__device__ __forceinline__ float df_diagonal2(const float *box)
+{
+    float d = 0.0f;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) d = fmaf(box[3 + c] - box[c], box[3 + c] - box[c], d);
+    return d;
+}
+
+__device__ __forceinline__ float df_radius2(const DfClass &k, float diag2)
+{
+    return fmaxf(k.floor2, kDfNear * kDfNear * diag2);
+}
+
+// h: the support in the caller's units, il = 1 / L.
+__device__ __forceinline__ DfClass df_classify(const float *tile, const DfHead &head, const DfTarget &tg,
+                                               bool live, double h, double il)
+{
+    DfClass k;
+    float at = 0.0f, ext2 = 0.0f;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        at = fmaxf(at, fabsf(tg.h[c]));
+        ext2 = fmaf(head.ext[c], head.ext[c], ext2);
+    }
+    const float hl = __double2float_ru(__dmul_rn(h, il)) * (1.0f + 0x1p-18f);
+    const int n_sub = (head.count + kDfSub - 1) / kDfSub;
+    k.floor2 = fmaxf(hl * hl * (1.0f + 0x1p-18f), ext2 * 0x1p-8f);
+    k.direct = 0;
+    k.close = 0;
+    k.rmin2 = 0x1p60f;
+    if (!(__all_sync(0xffffffffu, !live || at < kDfRange) && head.ok)) {
+        k.direct = (1u << n_sub) - 1u;
+        return k;
+    }
+    for (int q = 0; q < n_sub; ++q) {
+        const float *box = tile + kDfHeader + 6 * q;
+        float gap2 = 0.0f;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            float gap = fmaxf(box[c] - tg.h[c], tg.h[c] - box[3 + c]);
+            gap = fmaxf(0.0f, fmaf(-0x1p-20f, fabsf(tg.h[c]) + 1.0f, gap));
+            gap2 = fmaf(gap, gap, gap2);
+        }
+        gap2 *= 1.0f - 0x1p-18f;
+        const float diag2 = df_diagonal2(box), thr2 = df_radius2(k, diag2);
+        if (__any_sync(0xffffffffu, live && !(gap2 > thr2))) {
+            // (mostly softened pairs: no list)
+            if (hl * hl > 0.25f * diag2) {
+                k.direct |= 1u << q;
+                continue;
+            }
+            k.close |= 1u << q;
+        }
+        // (lanes without a target: any window)
+        if (live) k.rmin2 = fminf(k.rmin2, fmaxf(gap2, thr2 * (1.0f - 0x1p-10f)));
+    }
+    return k;
+}
+
+// The target's offset from a tile's centre in units of L.
+__device__ __forceinline__ double df_offset(const DfHead &head, const double c[3], const double x[3],
+                                            DfTarget &tg)
+{
+    const double il = pow2d(head.ok ? -head.el : 0);
+    const double xs[3] = {__dmul_rn(__dsub_rn(x[0], c[0]), il), __dmul_rn(__dsub_rn(x[1], c[1]), il),
+                          __dmul_rn(__dsub_rn(x[2], c[2]), il)};
+    df_split(xs, tg);
+    return il;
+}
+
+}  // namespace grav

@@ -46,6 +46,7 @@
 #pragma once
 
 #include "grav_common.cuh"
+#include "grav_df.cuh"
 
 namespace grav {
 
@@ -360,7 +361,7 @@ constexpr int kLoPlanes = 3;
 // when VOFF, else v); F64: tile = [S x D4 (x, m)][S x D4 (v, 0)].  Padding
 // sources have zero mass and sit far away, so they contribute exactly 0.
 // `mass` may be NULL (zero masses: the adjoint packs a_bar as "velocity").
-template <int S, bool MIXED, bool VOFF, bool PAIR = false>
+template <int S, bool MIXED, bool VOFF, bool PAIR = false, bool DF = false>
 __device__ __forceinline__ void pack_tile(int t, int64_t first, int64_t end,
                                           const double *__restrict__ pos,
                                           const double *__restrict__ vel,
@@ -453,6 +454,18 @@ __device__ __forceinline__ void pack_tile(int t, int64_t first, int64_t end,
         }
         tile[j] = pm;
         tile[S + j] = pv;
+    } else if (DF) {
+        const double off[3] = {__dsub_rn(x[0], cc[0]), __dsub_rn(x[1], cc[1]), __dsub_rn(x[2], cc[2])};
+        const double vo[3] = {__dsub_rn(v[0], (double)cvf[0]), __dsub_rn(v[1], (double)cvf[1]),
+                              __dsub_rn(v[2], (double)cvf[2])};
+        // half extents about the rounded centre
+        double half[3];
+#pragma unroll
+        for (int c = 0; c < 3; ++c)
+            half[c] = fmax(__dsub_ru(mm[2 * c + 1], cc[c]), __dsub_ru(cc[c], mm[2 * c]));
+        const double cmax = fmax(fabs(cc[0]), fmax(fabs(cc[1]), fabs(cc[2])));
+        df_pack<S>(static_cast<char *>(src) + (int64_t)t * df_stride<S>(), j, ok, (int)(end - first < S ? end - first : S),
+                   off, vo, m, half, cmax);
     } else {
         D4 *tile = static_cast<D4 *>(src) + (int64_t)t * 2 * S;
         D4 pm, pv;
@@ -481,7 +494,7 @@ __device__ __forceinline__ void pack_tile(int t, int64_t first, int64_t end,
 }
 
 // Single system: tile t holds sources [t*S, min((t+1)*S, n_src)).
-template <int S, bool MIXED, bool VOFF, bool PAIR = false>
+template <int S, bool MIXED, bool VOFF, bool PAIR = false, bool DF = false>
 __global__ void __launch_bounds__(S)
 pack_tiles_kernel(int64_t n_src, const double *__restrict__ pos, const double *__restrict__ vel,
                   const double *__restrict__ mass, TileGeom *__restrict__ geo, void *__restrict__ src,
@@ -489,8 +502,8 @@ pack_tiles_kernel(int64_t n_src, const double *__restrict__ pos, const double *_
 {
     const int64_t first = (int64_t)blockIdx.x * S;
     const int64_t end = first + S < n_src ? first + S : n_src;
-    pack_tile<S, MIXED, VOFF, PAIR>(blockIdx.x, first, end, pos, vel, mass, geo, src, flags,
-                                    src_lo);
+    pack_tile<S, MIXED, VOFF, PAIR, DF>(blockIdx.x, first, end, pos, vel, mass, geo, src, flags,
+                                        src_lo);
 }
 
 // ---------------------------------------------------------------------------
@@ -1817,7 +1830,7 @@ __device__ __forceinline__ int item_rank(const BatchView &b, int64_t ticket)
 
 // Batched packing: tile t belongs to the system s with
 // tile_off[s] <= t < tile_off[s + 1]; tiles never straddle two systems.
-template <int S, bool MIXED, bool VOFF, bool PAIR>
+template <int S, bool MIXED, bool VOFF, bool PAIR, bool DF = false>
 __global__ void __launch_bounds__(S)
 pack_tiles_batched_kernel(const BatchView b, const double *__restrict__ pos,
                           const double *__restrict__ vel, const double *__restrict__ mass,
@@ -1837,7 +1850,7 @@ pack_tiles_batched_kernel(const BatchView b, const double *__restrict__ pos,
     const int64_t first = b.sys[lo].offset + (int64_t)(t - b.tile_off[lo]) * S;
     const int64_t sys_end = b.sys[lo].offset + b.sys[lo].n;
     const int64_t end = first + S < sys_end ? first + S : sys_end;
-    pack_tile<S, MIXED, VOFF, PAIR>(t, first, end, pos, vel, mass, geo, src, flags, src_lo);
+    pack_tile<S, MIXED, VOFF, PAIR, DF>(t, first, end, pos, vel, mass, geo, src, flags, src_lo);
 }
 
 // ---------------------------------------------------------------------------
@@ -2390,7 +2403,8 @@ eval_mixed_batched_kernel(const EvalArgs a, const BatchView b)
 }
 
 // ---------------------------------------------------------------------------
-// K4: FP64 force kernel (one target per thread)
+// K4: FP64 force kernel of the periodic box and of adaptive softening (one
+// target per thread; open boundaries: grav_eval_df.cuh)
 // ---------------------------------------------------------------------------
 
 template <int S>
@@ -2428,14 +2442,10 @@ __device__ __forceinline__ bool f64_item(const EvalArgs &a, F64Smem<S> &sm, Ring
             hi[c] = __double2float_ru(xi[c]);
         }
     }
+    static_assert(MODE != kModeOpen, "open boundaries: df_item (grav_eval_df.cuh)");
     block_bbox<NT>(lo, hi, sm.blo, sm.bhi);
-    // open boundaries: each warp tests tiles against its own targets' box
-    // (lo/hi now hold it; the near and far loops synchronise nothing)
-    constexpr bool kWarpBox = MODE == kModeOpen;
-    const float blo_r[3] = {kWarpBox ? lo[0] : sm.blo[0], kWarpBox ? lo[1] : sm.blo[1],
-                            kWarpBox ? lo[2] : sm.blo[2]};
-    const float bhi_r[3] = {kWarpBox ? hi[0] : sm.bhi[0], kWarpBox ? hi[1] : sm.bhi[1],
-                            kWarpBox ? hi[2] : sm.bhi[2]};
+    const float blo_r[3] = {sm.blo[0], sm.blo[1], sm.blo[2]};
+    const float bhi_r[3] = {sm.bhi[0], sm.bhi[1], sm.bhi[2]};
     // periodic box: the target's close radius (close_radii; the FP64 pair
     // terms need no FP64 close field, only the runs)
     float rc2[1] = {-1.0f};
@@ -2488,11 +2498,9 @@ __device__ __forceinline__ bool f64_item(const EvalArgs &a, F64Smem<S> &sm, Ring
             const int cls = periodic_class<1>(tw, ti1, g, a.h2f_up, a.box_tie_f, rc2);
             close = __syncthreads_or((cls & 2) != 0) != 0;
             near = close || __syncthreads_or((cls & 1) != 0) != 0;
-        } else if (soft) {
+        } else {
             const float hm = fmaxf(h_block, a.geo_h[t]);
             near = tile_is_near(blo_r, bhi_r, g, __fmul_ru(hm, hm));
-        } else {
-            near = tile_is_near(blo_r, bhi_r, g, a.h2f_up);
         }
         const bool got = mbar_wait_bounded(&sm.bar[s], (ring.parity >> s) & 1u, a.flags);
         if (got)
@@ -2530,10 +2538,8 @@ __device__ __forceinline__ bool f64_item(const EvalArgs &a, F64Smem<S> &sm, Ring
             else if (periodic)
                 loop_d<S, POT, true, true>(sm.stage[s], sm.stage[s] + S, xi, i, g.first, h2, hinv,
                                            acc, a.box, a.box_inv, a.box_tie);
-            else if (!near)
-                loop_d<S, POT, false>(sm.stage[s], sm.stage[s] + S, xi, i, g.first, h2, hinv, acc);
             else
-                loop_d<S, POT, true>(sm.stage[s], sm.stage[s] + S, xi, i, g.first, h2, hinv, acc);
+                loop_d<S, POT, false>(sm.stage[s], sm.stage[s] + S, xi, i, g.first, h2, hinv, acc);
             target_velocity_d(acc, vr);
         }
 #pragma unroll
@@ -2711,11 +2717,16 @@ struct EvalConfig {
     int32_t threads, kt, s, unroll, sacc;
     eval_launch_fn launch[3][2];   // [mode][want_pot]
     occupancy_fn occupancy[3][2];
-    pack_launch_fn pack;
+    pack_launch_fn pack[3];        // [mode]
     batched_launch_fn launch_batched[2][2];   // [mode: open, periodic][want_pot]
     occupancy_fn occupancy_batched[2][2];
-    batched_pack_fn pack_batched;
+    batched_pack_fn pack_batched[2];
     bool paired;                   // mixed source tiles in the paired (FP32x2) layout
+    // FP64, open boundaries: the same on tiles of s sources (launch[0] and
+    // pack[0] take 2 s)
+    eval_launch_fn launch_fine[2] = {nullptr, nullptr};
+    occupancy_fn occupancy_fine[2] = {nullptr, nullptr};
+    pack_launch_fn pack_fine = nullptr;
 };
 
 template <int NT, int KT, int S, int MINB, int U, bool POT, bool SACC, bool PAIR, int MODE>
@@ -2764,12 +2775,12 @@ int occupancy_f64_batched(int *b)
     return (int)cudaOccupancyMaxActiveBlocksPerMultiprocessor(b, eval_f64_batched_kernel<NT, S, POT, MODE>, NT, 0);
 }
 
-template <int S, bool MIXED, bool VOFF, bool PAIR>
+template <int S, bool MIXED, bool VOFF, bool PAIR, bool DF = false>
 void launch_pack_batched(const BatchView &b, const double *pos, const double *vel, const double *mass,
                          TileGeom *geo, void *src, int32_t *flags, float *src_lo, int max_tiles,
                          cudaStream_t st)
 {
-    pack_tiles_batched_kernel<S, MIXED, VOFF, PAIR><<<max_tiles, S, 0, st>>>(b, pos, vel, mass, geo, src,
+    pack_tiles_batched_kernel<S, MIXED, VOFF, PAIR, DF><<<max_tiles, S, 0, st>>>(b, pos, vel, mass, geo, src,
                                                                             flags, src_lo);
 }
 
@@ -2785,11 +2796,11 @@ int occupancy_f64(int *b)
     return (int)cudaOccupancyMaxActiveBlocksPerMultiprocessor(b, eval_f64_kernel<NT, S, POT, MODE>, NT, 0);
 }
 
-template <int S, bool MIXED, bool VOFF, bool PAIR>
+template <int S, bool MIXED, bool VOFF, bool PAIR, bool DF = false>
 void launch_pack(int64_t n_src, const double *pos, const double *vel, const double *mass,
                  TileGeom *geo, void *src, int32_t *flags, float *src_lo, int n_tiles, cudaStream_t st)
 {
-    pack_tiles_kernel<S, MIXED, VOFF, PAIR><<<n_tiles, S, 0, st>>>(n_src, pos, vel, mass, geo, src, flags,
+    pack_tiles_kernel<S, MIXED, VOFF, PAIR, DF><<<n_tiles, S, 0, st>>>(n_src, pos, vel, mass, geo, src, flags,
                                                                   src_lo);
 }
 

@@ -125,10 +125,11 @@ void set_box(EvalArgs &a, double box)
     a.box_lo_f = box > 0.0 ? (float)(box - (double)a.box_f) : 0.0f;
 }
 
-int grid_for(const EvalConfig *c, int index, int mode, bool pot, int *grid)
+int grid_for(const EvalConfig *c, int index, int mode, bool fine, bool pot, int *grid)
 {
     static std::mutex mu;
-    static int cache[64][2][kMaxTileConfigs][3][2];   // [device][precision][config][mode][pot]
+    // [device][precision][config][mode, or 3: open on fine tiles][pot]
+    static int cache[64][2][kMaxTileConfigs][4][2];
     int dev = 0;
     int rc = check_cuda(cudaGetDevice(&dev), "cudaGetDevice");
     if (rc) return rc;
@@ -137,16 +138,43 @@ int grid_for(const EvalConfig *c, int index, int mode, bool pot, int *grid)
     if (rc) return rc;
     if (dev >= 64 || index >= kMaxTileConfigs) return fail(GRAV_ECUDA, "device or config index out of range");
     std::lock_guard<std::mutex> lk(mu);
-    int &slot = cache[dev][c->precision][index][mode][pot ? 1 : 0];
+    int &slot = cache[dev][c->precision][index][fine ? 3 : mode][pot ? 1 : 0];
     if (slot == 0) {
         int b = 0;
-        rc = check_cuda((cudaError_t)c->occupancy[mode][pot ? 1 : 0](&b), "cudaOccupancyMaxActiveBlocksPerMultiprocessor");
+        const occupancy_fn occ = fine ? c->occupancy_fine[pot ? 1 : 0] : c->occupancy[mode][pot ? 1 : 0];
+        rc = check_cuda((cudaError_t)occ(&b), "cudaOccupancyMaxActiveBlocksPerMultiprocessor");
         if (rc) return rc;
         if (b < 1) return fail(GRAV_ECUDA, "force kernel cannot be resident on an SM");
         slot = b * sms;
     }
     *grid = slot;
     return GRAV_OK;
+}
+
+// The open FP64 kernel (grav_eval_df.cuh) packs its tiles in two-part FP32,
+// twice the configuration's sources to a tile.  Where that leaves fewer work
+// items (target block x tile) than two rounds of the resident CTAs and the
+// sources may be split over them, the items count more than the cost per tile:
+// tiles of the configuration's size (2011 elements 592 -> 470 us; 12289 elements
+// 3.4 ms with the large tiles, 4.2 ms with the small ones).
+constexpr int64_t kFinePairs = 1LL << 25;
+
+bool fine_tiles(const grav_params *p, const EvalConfig *c, int mode, int64_t n_src, int64_t n_idx_max)
+{
+    return c->precision == GRAV_F64 && mode == kModeOpen && p->max_split != 1 &&
+           n_src * n_idx_max < kFinePairs;
+}
+
+// Sources per packed tile and bytes per source of the packed tiles.
+int64_t tile_sources(const EvalConfig *c, int mode, bool fine)
+{
+    return c->precision == GRAV_F64 && mode == kModeOpen && !fine ? 2 * c->s : c->s;
+}
+
+int64_t source_bytes(const EvalConfig *c, int mode)
+{
+    if (c->precision == GRAV_MIXED) return 32;
+    return mode == kModeOpen ? kDfBytesPerSource : 64;
 }
 
 struct Layout {
@@ -158,20 +186,20 @@ struct Layout {
 };
 
 int make_layout(const grav_params *p, const EvalConfig *c, int64_t n_src, int64_t n_idx_max,
-                Layout *L, bool soft = false)
+                Layout *L, int mode)
 {
+    const bool soft = mode == kModeSoft;
     int sms = 0;
     int rc = device_sm_count(&sms);
     if (rc) return rc;
-    const int64_t S = c->s;
+    const int64_t S = tile_sources(c, mode, fine_tiles(p, c, mode, n_src, n_idx_max));
     const int64_t BT = (int64_t)c->threads * c->kt;
-    const int64_t elem = (c->precision == GRAV_MIXED) ? 16 : 32;
     const int NC = p->want_pot ? kNCPot : kNC;
     L->max_split = p->max_split > 0 ? p->max_split : kDefaultMaxSplit;
     L->n_tiles = (n_src + S - 1) / S;
     L->geo_off = 0;
     L->src_off = round_up(L->n_tiles * (int64_t)sizeof(TileGeom), 256);
-    L->lo_off = L->src_off + round_up(L->n_tiles * 2 * S * elem, 256);
+    L->lo_off = L->src_off + round_up(L->n_tiles * S * source_bytes(c, mode), 256);
     const int64_t lo_bytes = (c->precision == GRAV_MIXED) ? L->n_tiles * kLoPlanes * S * 4 : 0;
     L->part_off = L->lo_off + round_up(lo_bytes, 256);
     const int64_t n_tb_max = (n_idx_max + BT - 1) / BT;
@@ -245,7 +273,7 @@ int64_t workspace_bytes_for(const grav_params *p, int64_t n_src, int64_t n_idx_m
     const int mode = soft ? kModeSoft : (p->box > 0.0 ? kModePeriodic : kModeOpen);
     const EvalConfig *c = resolve(p, mode, n_idx_max, &index);
     Layout L;
-    rc = make_layout(p, c, n_src, n_idx_max, &L, soft);
+    rc = make_layout(p, c, n_src, n_idx_max, &L, mode);
     if (rc) return rc;
     return L.total;
 }
@@ -276,14 +304,15 @@ int eval_single(const char *who, const grav_params *p, bool soft, int64_t n_src,
     int index = 0;
     const EvalConfig *c = resolve(p, mode, n_idx_max, &index);
     Layout L;
-    rc = make_layout(p, c, n_src, n_idx_max, &L, soft);
+    rc = make_layout(p, c, n_src, n_idx_max, &L, mode);
     if (rc) return rc;
     if (workspace_bytes < L.total)
         return fail(GRAV_ENOMEM, "%s: workspace of %lld bytes < %lld", who, (long long)workspace_bytes,
                     (long long)L.total);
     const bool want_pot = p->want_pot != 0;
     int grid = 0;
-    rc = grid_for(c, index, mode, want_pot, &grid);
+    const bool fine = fine_tiles(p, c, mode, n_src, n_idx_max);
+    rc = grid_for(c, index, mode, fine, want_pot, &grid);
     if (rc) return rc;
 
     char *ws = static_cast<char *>(workspace);
@@ -330,7 +359,7 @@ int eval_single(const char *who, const grav_params *p, bool soft, int64_t n_src,
     }
 
     cudaStream_t st = as_stream(stream);
-    c->pack(n_src, pos, vel, mass, const_cast<TileGeom *>(a.geo), const_cast<void *>(a.src), flags_dev,
+    (fine ? c->pack_fine : c->pack[mode])(n_src, pos, vel, mass, const_cast<TileGeom *>(a.geo), const_cast<void *>(a.src), flags_dev,
             const_cast<float *>(a.src_lo), (int)L.n_tiles, st);
     rc = check_launch("grav_eval/pack");
     if (rc) return rc;
@@ -341,7 +370,7 @@ int eval_single(const char *who, const grav_params *p, bool soft, int64_t n_src,
         rc = check_launch("grav_eval_soft/pack_soft");
         if (rc) return rc;
     }
-    c->launch[mode][want_pot ? 1 : 0](a, grid, st);
+    (fine ? c->launch_fine : c->launch[mode])[want_pot ? 1 : 0](a, grid, st);
     rc = check_launch("grav_eval/eval");
     if (rc) return rc;
     const int32_t BT = c->threads * c->kt;
@@ -518,11 +547,10 @@ struct BatchLayout {
     int64_t max_tiles;
 };
 
-BatchLayout batch_layout(const EvalConfig *c, int32_t n_sys, int64_t n_total)
+BatchLayout batch_layout(const EvalConfig *c, int mode, int32_t n_sys, int64_t n_total)
 {
     BatchLayout L;
-    const int64_t S = c->s;
-    const int64_t elem = (c->precision == GRAV_MIXED) ? 16 : 32;
+    const int64_t S = tile_sources(c, mode, false);
     L.max_tiles = (n_total + S - 1) / S + n_sys;
     int64_t o = 0;
     L.hdr = o;
@@ -542,7 +570,7 @@ BatchLayout batch_layout(const EvalConfig *c, int32_t n_sys, int64_t n_total)
     L.geo = o;
     o += round_up(L.max_tiles * (int64_t)sizeof(TileGeom), 256);
     L.src = o;
-    o += round_up(L.max_tiles * 2 * S * elem, 256);
+    o += round_up(L.max_tiles * S * source_bytes(c, mode), 256);
     L.lo = o;
     o += round_up((c->precision == GRAV_MIXED) ? L.max_tiles * kLoPlanes * S * 4 : 0, 256);
     L.total = o;
@@ -603,7 +631,7 @@ extern "C" int64_t grav_batched_workspace_bytes(const grav_params *p, int32_t n_
         return fail(GRAV_EINVAL, "grav_batched_workspace_bytes: n_sys or n_total out of range");
     int index = 0;
     const EvalConfig *c = resolve_batched(p, &index);
-    return batch_layout(c, n_sys, n_total).total;
+    return batch_layout(c, p->box > 0.0 ? kModePeriodic : kModeOpen, n_sys, n_total).total;
 }
 
 extern "C" int grav_eval_batched(const grav_params *p, int32_t n_sys, const grav_system *systems,
@@ -628,7 +656,8 @@ extern "C" int grav_eval_batched(const grav_params *p, int32_t n_sys, const grav
         return fail(GRAV_EINVAL, "%s: workspace missing or not 256-byte aligned", who);
     int index = 0;
     const EvalConfig *c = resolve_batched(p, &index);
-    const BatchLayout L = batch_layout(c, n_sys, n_total);
+    const int mode = p->box > 0.0 ? kModePeriodic : kModeOpen;
+    const BatchLayout L = batch_layout(c, mode, n_sys, n_total);
     if (workspace_bytes < L.total)
         return fail(GRAV_ENOMEM, "%s: workspace of %lld bytes < %lld", who, (long long)workspace_bytes,
                     (long long)L.total);
@@ -688,9 +717,10 @@ extern "C" int grav_eval_batched(const grav_params *p, int32_t n_sys, const grav
 
     cudaStream_t st = as_stream(stream);
     const int32_t BT = c->threads * c->kt;
-    rc = launch_batch_plan(b, idx, n_idx_dev, n_idx_max, n_total, c->s, BT, p->box, flags_dev, st);
+    rc = launch_batch_plan(b, idx, n_idx_dev, n_idx_max, n_total,
+                           (int32_t)tile_sources(c, mode, false), BT, p->box, flags_dev, st);
     if (rc) return rc;
-    c->pack_batched(b, pos, vel, mass, const_cast<TileGeom *>(a.geo), const_cast<void *>(a.src),
+    c->pack_batched[p->box > 0.0 ? 1 : 0](b, pos, vel, mass, const_cast<TileGeom *>(a.geo), const_cast<void *>(a.src),
                     flags_dev, const_cast<float *>(a.src_lo), (int)L.max_tiles, st);
     rc = check_launch("grav_eval_batched/pack");
     if (rc) return rc;

@@ -30,10 +30,11 @@ GRAV_MIXED_CONFIG_LIST(GRAV_MIXED_EXTERN)
     {GRAV_MIXED, NT, KT, S, U, SACC,                                                          \
      GRAV_MIXED_FN3(launch_mixed, NT, KT, S, MINB, U, SACC, PAIR),                            \
      GRAV_MIXED_FN3(occupancy_mixed, NT, KT, S, MINB, U, SACC, PAIR),                         \
-     launch_pack<S, true, true, PAIR>,                                                        \
+     {launch_pack<S, true, true, PAIR>, launch_pack<S, true, true, PAIR>,                     \
+      launch_pack<S, true, true, PAIR>},                                                      \
      GRAV_MIXED_FN2(launch_mixed_batched, NT, KT, S, MINB, U, SACC, PAIR),                    \
      GRAV_MIXED_FN2(occupancy_mixed_batched, NT, KT, S, MINB, U, SACC, PAIR),                 \
-     launch_pack_batched<S, true, true, PAIR>, PAIR},
+     {launch_pack_batched<S, true, true, PAIR>, launch_pack_batched<S, true, true, PAIR>}, PAIR},
 
 static const EvalConfig kMixedConfigs[] = {GRAV_MIXED_CONFIG_LIST(GRAV_MIXED_CFG)};
 static_assert(sizeof(kMixedConfigs) / sizeof(kMixedConfigs[0]) <= kMaxTileConfigs,
