@@ -14,14 +14,23 @@
 //
 // One thread per element, 128 per CTA.  Sources are packed once into tiles
 // of 128: FP64 position and mass, FP32 offsets from the tile's centre, and an
-// outward-rounded FP32 bounding box.  In every pass a CTA tests all tile boxes
-// against its own box grown by the largest support still iterating (one tile
-// per thread, compacted by ballot); for each such tile a thread skips it when
-// its own element is farther than h from the box, and otherwise pre-filters
-// every source with an FP32 distance test that carries an explicit bound on
-// its rounding, so the FP64 sums (the distance test that decides, W, dW/dh,
-// dpsi/dh) run only for candidate neighbours.  Newton steps are limited to a
-// factor of 2 in h.  Every loop is bounded by max_iter passes.
+// outward-rounded FP32 bounding box.  A scan of the sources tests all tile boxes
+// against the CTA's box grown by the largest radius in search (one tile per
+// thread, compacted by ballot); for each such tile a thread skips it when its
+// own element is farther than its radius from the box, and otherwise
+// pre-filters every source with an FP32 distance test that carries an explicit
+// bound on its rounding.  What passes is listed, with its FP64 distance, up to
+// 1.25 times the support, and the Newton passes run over the lists: a scan is
+// repeated only for supports that outgrow their list.  In each pass a thread
+// first collects the listed sources inside its support (integer compares of
+// the FP64 bits), then sums W, dW/dh and dpsi/dh over them, so the lanes of a
+// warp run the FP64 terms side by side: FP64 bounds this kernel, and with the
+// terms inside the scan a warp ran them once for every source inside any of
+// its 32 supports, 12 lanes active (40961 elements, n_ngb = 32, guesses off by
+// up to 20%: 8.1 ms, with the lists 4.1 ms).  An element with more than
+// kSoftList sources in reach sums them in the scans.  Every order of summation
+// is that of the sources.  Newton steps are limited to a factor of 2 in h.
+// Every loop is bounded by max_iter passes.
 #include <cmath>
 
 #include "grav_common.cuh"
@@ -183,6 +192,9 @@ __device__ __forceinline__ bool box_near(const float blo[3], const float bhi[3],
     return d2 < __fmul_ru(H, H);
 }
 
+constexpr int kSoftList = 224;      // listed sources per element
+constexpr double kSoftReach = 1.25; // list radius over the support it is made for
+
 __global__ void __launch_bounds__(kSoftNT) soft_solve_kernel(SoftArgs a)
 {
     __shared__ double4 sx[kSoftS];
@@ -209,109 +221,163 @@ __global__ void __launch_bounds__(kSoftNT) soft_solve_kernel(SoftArgs a)
     int32_t it = 0;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const float inf = __int_as_float(0x7f800000);
+    // the list: sources within `reach` in ascending order, and their FP64
+    // squared distances and distances
+    int32_t nj[kSoftList];
+    double nr2[kSoftList], nr[kSoftList];
+    int cnt = 0;
+    double reach = 0.0;
+    bool direct = false;      // more sources in reach than the list holds
 
     for (int pass = 0; pass < a.max_iter; ++pass) {
-        // ---- the CTA's box and largest support over the elements still iterating ----
-        float l[3], u[3], hm = done ? 0.0f : __double2float_ru(h);
-        for (int c = 0; c < 3; ++c) {
-            l[c] = done ? inf : __double2float_rd(xi[c]);
-            u[c] = done ? -inf : __double2float_ru(xi[c]);
-        }
-        for (int o = 16; o > 0; o >>= 1) {
-            hm = fmaxf(hm, __shfl_xor_sync(0xffffffffu, hm, o));
-            for (int c = 0; c < 3; ++c) {
-                l[c] = fminf(l[c], __shfl_xor_sync(0xffffffffu, l[c], o));
-                u[c] = fmaxf(u[c], __shfl_xor_sync(0xffffffffu, u[c], o));
-            }
-        }
-        if (lane == 0) {
-            rh[wid] = hm;
-            for (int c = 0; c < 3; ++c) {
-                rlo[c][wid] = l[c];
-                rhi[c][wid] = u[c];
-            }
-        }
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            float H = 0.0f;
-            float L[3] = {inf, inf, inf}, U[3] = {-inf, -inf, -inf};
-            for (int w = 0; w < kSoftNT / 32; ++w) {
-                H = fmaxf(H, rh[w]);
-                for (int c = 0; c < 3; ++c) {
-                    L[c] = fminf(L[c], rlo[c][w]);
-                    U[c] = fmaxf(U[c], rhi[c][w]);
-                }
-            }
-            bh = H;
-            for (int c = 0; c < 3; ++c) {
-                blo[c] = L[c];
-                bhi[c] = U[c];
-            }
-        }
-        __syncthreads();
-        if (!(bh > 0.0f)) break;                 // every element of the CTA is done
-        const float B_lo[3] = {blo[0], blo[1], blo[2]}, B_hi[3] = {bhi[0], bhi[1], bhi[2]};
-        const float H = bh;
-
-        // ---- sums at the current supports over the tiles that can reach ----
+        if (!__syncthreads_or(!done)) break;       // every element of the CTA is done
         double rho = 0.0, rho_h = 0.0, psi_h = 0.0;
         const double hinv = 1.0 / h, h2 = h * h;
-        const float hf = __double2float_ru(h);
-        const float hlim2 = __fmul_ru(hf, hf);
-        for (int64_t t0 = 0; t0 < a.n_tiles; t0 += kSoftNT) {
-            const int64_t tt = t0 + threadIdx.x;
-            const bool near = tt < a.n_tiles && box_near(B_lo, B_hi, a.box[tt], H);
-            const uint32_t bal = __ballot_sync(0xffffffffu, near);
-            if (lane == 0) wcount[wid] = __popc(bal);
-            __syncthreads();
-            int base = 0, total = 0;
-            for (int w = 0; w < kSoftNT / 32; ++w) {
-                if (w < wid) base += wcount[w];
-                total += wcount[w];
+        // ---- scans: lists for the supports that outgrew theirs, the sums of
+        // the elements without a list (a second scan when a list overflows)
+        bool want = !done && (direct || h > reach);
+        while (__syncthreads_or(want)) {
+            const double rad = direct ? h : kSoftReach * h;
+            float l[3], u[3], hm = want ? __double2float_ru(rad) : 0.0f;
+            for (int c = 0; c < 3; ++c) {
+                l[c] = want ? __double2float_rd(xi[c]) : inf;
+                u[c] = want ? __double2float_ru(xi[c]) : -inf;
             }
-            if (near) list[base + __popc(bal & ((1u << lane) - 1u))] = (int32_t)(tt - t0);
+            for (int o = 16; o > 0; o >>= 1) {
+                hm = fmaxf(hm, __shfl_xor_sync(0xffffffffu, hm, o));
+                for (int c = 0; c < 3; ++c) {
+                    l[c] = fminf(l[c], __shfl_xor_sync(0xffffffffu, l[c], o));
+                    u[c] = fmaxf(u[c], __shfl_xor_sync(0xffffffffu, u[c], o));
+                }
+            }
+            if (lane == 0) {
+                rh[wid] = hm;
+                for (int c = 0; c < 3; ++c) {
+                    rlo[c][wid] = l[c];
+                    rhi[c][wid] = u[c];
+                }
+            }
             __syncthreads();
-            for (int k = 0; k < total; ++k) {
-                const int64_t t = t0 + list[k];
-                sx[threadIdx.x] = a.src[t * kSoftS + threadIdx.x];   // kSoftNT == kSoftS
-                sx32[threadIdx.x] = a.src32[t * kSoftS + threadIdx.x];
-                const SoftBox tb = a.box[t];
-                __syncthreads();
-                if (!done) {
-                    // own offset from the tile centre (FP64, rounded once) and
-                    // a lower bound of the distance to the tile's box
-                    float tq[3], tmax = 0.0f, gap2 = 0.0f;
+            if (threadIdx.x == 0) {
+                float H = 0.0f;
+                float L[3] = {inf, inf, inf}, U[3] = {-inf, -inf, -inf};
+                for (int w = 0; w < kSoftNT / 32; ++w) {
+                    H = fmaxf(H, rh[w]);
                     for (int c = 0; c < 3; ++c) {
-                        tq[c] = __double2float_rn(xi[c] - tb.c[c]);
-                        tmax = fmaxf(tmax, fabsf(tq[c]));
-                        const float gap = fmaxf(0.0f, __fsub_rd(__fsub_rd(fabsf(tq[c]), tb.ext),
-                                                                 __fmul_ru(fabsf(tq[c]), 0x1p-22f)));
-                        gap2 = __fmaf_rd(gap, gap, gap2);
+                        L[c] = fminf(L[c], rlo[c][w]);
+                        U[c] = fmaxf(U[c], rhi[c][w]);
                     }
-                    if (gap2 < hlim2) {
-                        // |d32 - d| <= err per component: both offsets were
-                        // rounded once and their difference once more
-                        const float err = __fmul_ru(__fadd_ru(tb.ext, tmax), 0x1p-21f);
-                        const float hl = __fadd_ru(hf, __fmul_ru(err, 1.8f));
-                        const float lim = __fmul_ru(__fmul_ru(hl, hl), 1.0f + 0x1p-20f);
-                        for (int j = 0; j < kSoftS; ++j) {
-                            const float4 q = sx32[j];
-                            const float ex = q.x - tq[0], ey = q.y - tq[1], ez = q.z - tq[2];
-                            if (fmaf(ex, ex, fmaf(ey, ey, ez * ez)) >= lim) continue;
-                            const double4 s = sx[j];
-                            const double dx = s.x - xi[0], dy = s.y - xi[1], dz = s.z - xi[2];
-                            const double r2 = fma(dx, dx, fma(dy, dy, dz * dz));
-                            if (r2 < h2) {
-                                double w, wh, ph;
-                                density_terms(sqrt(r2) * hinv, hinv, w, wh, ph);
-                                rho = fma(s.w, w, rho);
-                                rho_h = fma(s.w, wh, rho_h);
-                                if (t * kSoftS + j != i) psi_h = fma(s.w, ph, psi_h);
+                }
+                bh = H;
+                for (int c = 0; c < 3; ++c) {
+                    blo[c] = L[c];
+                    bhi[c] = U[c];
+                }
+            }
+            __syncthreads();
+            const float B_lo[3] = {blo[0], blo[1], blo[2]}, B_hi[3] = {bhi[0], bhi[1], bhi[2]};
+            const float H = bh;
+            const bool any_direct = __syncthreads_or(want && direct) != 0;
+            if (want && !direct) cnt = 0;
+            const float hf = __double2float_ru(rad);
+            const float hlim2 = __fmul_ru(hf, hf);
+            for (int64_t t0 = 0; t0 < a.n_tiles; t0 += kSoftNT) {
+                const int64_t tt = t0 + threadIdx.x;
+                const bool near = tt < a.n_tiles && box_near(B_lo, B_hi, a.box[tt], H);
+                const uint32_t bal = __ballot_sync(0xffffffffu, near);
+                if (lane == 0) wcount[wid] = __popc(bal);
+                __syncthreads();
+                int base = 0, total = 0;
+                for (int w = 0; w < kSoftNT / 32; ++w) {
+                    if (w < wid) base += wcount[w];
+                    total += wcount[w];
+                }
+                if (near) list[base + __popc(bal & ((1u << lane) - 1u))] = (int32_t)(tt - t0);
+                __syncthreads();
+                for (int k = 0; k < total; ++k) {
+                    const int64_t t = t0 + list[k];
+                    if (any_direct) sx[threadIdx.x] = a.src[t * kSoftS + threadIdx.x];   // kSoftNT == kSoftS
+                    sx32[threadIdx.x] = a.src32[t * kSoftS + threadIdx.x];
+                    const SoftBox tb = a.box[t];
+                    __syncthreads();
+                    if (want) {
+                        // own offset from the tile centre (FP64, rounded once) and
+                        // a lower bound of the distance to the tile's box
+                        float tq[3], tmax = 0.0f, gap2 = 0.0f;
+                        for (int c = 0; c < 3; ++c) {
+                            tq[c] = __double2float_rn(xi[c] - tb.c[c]);
+                            tmax = fmaxf(tmax, fabsf(tq[c]));
+                            const float gap = fmaxf(0.0f, __fsub_rd(__fsub_rd(fabsf(tq[c]), tb.ext),
+                                                                     __fmul_ru(fabsf(tq[c]), 0x1p-22f)));
+                            gap2 = __fmaf_rd(gap, gap, gap2);
+                        }
+                        if (gap2 < hlim2) {
+                            // |d32 - d| <= err per component: both offsets were
+                            // rounded once and their difference once more
+                            const float err = __fmul_ru(__fadd_ru(tb.ext, tmax), 0x1p-21f);
+                            const float hl = __fadd_ru(hf, __fmul_ru(err, 1.8f));
+                            const float lim = __fmul_ru(__fmul_ru(hl, hl), 1.0f + 0x1p-20f);
+#pragma unroll 4
+                            for (int j = 0; j < kSoftS; ++j) {
+                                const float4 q = sx32[j];
+                                const float ex = q.x - tq[0], ey = q.y - tq[1], ez = q.z - tq[2];
+                                if (fmaf(ex, ex, fmaf(ey, ey, ez * ez)) >= lim) continue;
+                                if (!direct) {
+                                    if (cnt < kSoftList) nj[cnt] = (int32_t)(t * kSoftS + j);
+                                    ++cnt;
+                                    continue;
+                                }
+                                const double4 s = sx[j];
+                                const double dx = s.x - xi[0], dy = s.y - xi[1], dz = s.z - xi[2];
+                                const double r2 = fma(dx, dx, fma(dy, dy, dz * dz));
+                                if (r2 < h2) {
+                                    double w, wh, ph;
+                                    density_terms(sqrt(r2) * hinv, hinv, w, wh, ph);
+                                    rho = fma(s.w, w, rho);
+                                    rho_h = fma(s.w, wh, rho_h);
+                                    if (t * kSoftS + j != i) psi_h = fma(s.w, ph, psi_h);
+                                }
                             }
                         }
                     }
+                    __syncthreads();
                 }
-                __syncthreads();
+            }
+            if (want) {
+                if (!direct && cnt > kSoftList) {
+                    direct = true;                 // sum this pass in another scan
+                } else {
+                    want = false;
+                    if (!direct) {
+                        reach = rad;
+                        for (int k = 0; k < cnt; ++k) {
+                            const double4 s = a.src[nj[k]];
+                            const double dx = s.x - xi[0], dy = s.y - xi[1], dz = s.z - xi[2];
+                            const double r2 = fma(dx, dx, fma(dy, dy, dz * dz));
+                            nr2[k] = r2;
+                            nr[k] = sqrt(r2);
+                        }
+                    }
+                }
+            }
+        }
+
+        // ---- sums over the listed sources inside the support ----
+        if (!done && !direct) {
+            uint8_t in[kSoftList];
+            int n_in = 0;
+            const long long h2b = __double_as_longlong(h2);      // (non-negative: ordered as integers)
+            for (int k = 0; k < cnt; ++k)
+                if (__double_as_longlong(nr2[k]) < h2b) in[n_in++] = (uint8_t)k;
+            for (int q = 0; q < n_in; ++q) {
+                const int k = in[q];
+                const int32_t j = nj[k];
+                const double m = a.mass[j];
+                double w, wh, ph;
+                density_terms(nr[k] * hinv, hinv, w, wh, ph);
+                rho = fma(m, w, rho);
+                rho_h = fma(m, wh, rho_h);
+                if (j != i) psi_h = fma(m, ph, psi_h);
             }
         }
 
