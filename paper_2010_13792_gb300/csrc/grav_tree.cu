@@ -9,7 +9,7 @@
 //     * 2^21) clamped to [0, 2^21 - 1]; 63-bit keys interleaving x, y, z from
 //     the highest bit down;
 //   - order: elements sorted by (key, index) -- a stable LSD radix sort of
-//     the keys over the index order (16 passes of 4 bits);
+//     the keys over the index order (8 passes of 8 bits);
 //   - nodes: a node at level l holds the run of elements that share the top
 //     3l key bits and has side ext 2^-l; it is a leaf when it holds at most
 //     leaf_size elements or l = 21, else its non-empty octants are its
@@ -24,9 +24,9 @@
 //     its mean velocity, a leaf that is not accepted is summed element by
 //     element (j != i), any other node is opened; children in octant order.
 // Building: per level, one thread per node finds its octant runs by binary
-// search and appends its children with one atomic add (node numbers vary
-// from run to run, the tree and the walk order do not); moments bottom-up and
-// the "next" links top-down, level by level.  The walk is stackless: after a
+// search, appends its children with one atomic add (node numbers vary from run
+// to run, the tree and the walk order do not) and links them ("next"); moments
+// bottom-up, level by level.  The walk is stackless: after a
 // node is accepted or a leaf is summed the walk continues at the node's next
 // link (its next sibling, else its parent's next link).  GRAV_F64: pair terms
 // as in the FP64 direct kernel, sums compensated every 32 interactions;
@@ -42,8 +42,9 @@ constexpr int kMaxLevel = 21;
 constexpr int kSortNT = 256;
 constexpr int kSortPer = 16;                    // items per thread
 constexpr int kSortBlock = kSortNT * kSortPer;  // 4096 items per CTA
-constexpr int kBins = 16;                       // 4-bit digits
-constexpr int kPasses = 16;
+constexpr int kBins = 256;                      // 8-bit digits
+constexpr int kPasses = 8;
+constexpr int kSortWarps = kSortNT / 32;
 constexpr int kBboxBlocks = 1024;
 constexpr int kWalkNT = 128;
 constexpr int kFlushEvery = 32;
@@ -55,7 +56,7 @@ struct TreeView {
     uint64_t *key;        // sorted keys (after the sort)
     int32_t *order;       // sorted element indices
     double *frame;        // lo[3], ext
-    int32_t *counters;    // [0] nodes, [1 + l] first node of level l (l = 0..23)
+    int32_t *counters;    // [0] nodes, [1 + l] first node of level l, [32 + l] nodes of level l (l = 0..23)
     int32_t *first, *count, *child_first, *next;
     int8_t *n_child, *level;
     double *m, *com, *vcom;
@@ -99,7 +100,7 @@ TreeLayout tree_layout(int64_t n, int32_t leaf)
     L.hist = take(nb * kBins * 4);
     L.part = take(kBboxBlocks * 6 * 8);
     L.frame = take(4 * 8);
-    L.counters = take(32 * 4);
+    L.counters = take(64 * 4);
     L.first = take(mn * 4);
     L.count = take(mn * 4);
     L.child_first = take(mn * 4);
@@ -122,54 +123,72 @@ TreeLayout tree_layout(int64_t n, int32_t leaf)
 // Bounding cube and keys
 // ---------------------------------------------------------------------------
 
-__global__ void __launch_bounds__(256) bbox_partial_kernel(int64_t n, const double *__restrict__ pos,
-                                                           double *__restrict__ part)
+// Smallest and largest coordinates as integer order keys (FP64 compares run at
+// 1/64 of the integer rate): part[2 c] and part[2 c + 1] of each CTA.  NaN
+// coordinates are left out.
+__device__ __forceinline__ void bbox_block(long long lo[3], long long hi[3], long long *out)
 {
-    __shared__ double s[6][8];
-    const double inf = __longlong_as_double(0x7ff0000000000000LL);
-    double lo[3] = {inf, inf, inf}, hi[3] = {-inf, -inf, -inf};
-    for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < n; i += (int64_t)gridDim.x * 256)
-        for (int c = 0; c < 3; ++c) {
-            const double x = pos[3 * i + c];
-            lo[c] = fmin(lo[c], x);
-            hi[c] = fmax(hi[c], x);
-        }
-    for (int c = 0; c < 3; ++c)
-        for (int o = 16; o > 0; o >>= 1) {
-            lo[c] = fmin(lo[c], __shfl_xor_sync(0xffffffffu, lo[c], o));
-            hi[c] = fmax(hi[c], __shfl_xor_sync(0xffffffffu, hi[c], o));
-        }
+    __shared__ long long s[6][8];
+    for (int c = 0; c < 3; ++c) {
+        lo[c] = warp_min_key(lo[c]);
+        hi[c] = ~warp_min_key(~hi[c]);
+    }
     if ((threadIdx.x & 31) == 0)
         for (int c = 0; c < 3; ++c) {
-            s[c][threadIdx.x >> 5] = lo[c];
-            s[3 + c][threadIdx.x >> 5] = hi[c];
+            s[2 * c][threadIdx.x >> 5] = lo[c];
+            s[2 * c + 1][threadIdx.x >> 5] = hi[c];
         }
     __syncthreads();
     if (threadIdx.x < 6) {
-        double v = s[threadIdx.x][0];
-        for (int w = 1; w < 8; ++w)
-            v = threadIdx.x < 3 ? fmin(v, s[threadIdx.x][w]) : fmax(v, s[threadIdx.x][w]);
-        part[(int64_t)blockIdx.x * 6 + threadIdx.x] = v;
+        long long v = s[threadIdx.x][0];
+        for (int w = 1; w < 8; ++w) {
+            const long long k = s[threadIdx.x][w];
+            if ((threadIdx.x & 1) ? k > v : k < v) v = k;
+        }
+        out[threadIdx.x] = v;
     }
+    __syncthreads();
 }
 
-__global__ void bbox_final_kernel(int nb, const double *__restrict__ part, double *__restrict__ frame)
+constexpr long long kKeyInf = 0x7ff0000000000000LL;     // the key of +inf; ~ of it is that of -inf
+
+__global__ void __launch_bounds__(256) bbox_partial_kernel(int64_t n, const double *__restrict__ pos,
+                                                           long long *__restrict__ part)
 {
-    if (threadIdx.x != 0) return;
-    const double inf = __longlong_as_double(0x7ff0000000000000LL);
-    double lo[3] = {inf, inf, inf}, hi[3] = {-inf, -inf, -inf};
-    for (int b = 0; b < nb; ++b)
+    long long lo[3] = {kKeyInf, kKeyInf, kKeyInf}, hi[3] = {~kKeyInf, ~kKeyInf, ~kKeyInf};
+    for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < n; i += (int64_t)gridDim.x * 256)
         for (int c = 0; c < 3; ++c) {
-            lo[c] = fmin(lo[c], part[6 * b + c]);
-            hi[c] = fmax(hi[c], part[6 * b + 3 + c]);
+            const double x = pos[3 * i + c];
+            if ((__double_as_longlong(x) & 0x7fffffffffffffffLL) > kKeyInf) continue;   // NaN
+            const long long k = order_key(x);
+            lo[c] = k < lo[c] ? k : lo[c];
+            hi[c] = k > hi[c] ? k : hi[c];
         }
+    bbox_block(lo, hi, part + 6 * (int64_t)blockIdx.x);
+}
+
+// One CTA of 256: the cube from the partial boxes (one thread took 0.42 ms
+// over 1024 of them).
+__global__ void __launch_bounds__(256) bbox_final_kernel(int nb, const long long *__restrict__ part,
+                                                         double *__restrict__ frame)
+{
+    __shared__ long long all[6];
+    long long lo[3] = {kKeyInf, kKeyInf, kKeyInf}, hi[3] = {~kKeyInf, ~kKeyInf, ~kKeyInf};
+    for (int b = threadIdx.x; b < nb; b += 256)
+        for (int c = 0; c < 3; ++c) {
+            const long long l = part[6 * b + 2 * c], h = part[6 * b + 2 * c + 1];
+            lo[c] = l < lo[c] ? l : lo[c];
+            hi[c] = h > hi[c] ? h : hi[c];
+        }
+    bbox_block(lo, hi, all);
+    if (threadIdx.x != 0) return;
     double ext = 0.0;
     for (int c = 0; c < 3; ++c) {
-        const double e = __dsub_rn(hi[c], lo[c]);
+        const double e = __dsub_rn(order_value(all[2 * c + 1]), order_value(all[2 * c]));
         if (e > ext) ext = e;
     }
     if (!(ext > 0.0)) ext = 1.0;
-    for (int c = 0; c < 3; ++c) frame[c] = lo[c];
+    for (int c = 0; c < 3; ++c) frame[c] = order_value(all[2 * c]);
     frame[3] = ext;
 }
 
@@ -203,7 +222,11 @@ __global__ void __launch_bounds__(256) key_kernel(int64_t n, const double *__res
 }
 
 // ---------------------------------------------------------------------------
-// Stable LSD radix sort of (key, index), 4-bit digits
+// Stable LSD radix sort of (key, index), 8-bit digits.  Per pass: digit counts
+// of every CTA's 4096 keys, one scan of the counts, then each CTA ranks its keys
+// -- a warp takes 512 consecutive keys, 32 at a time, and the lanes that hold
+// the same digit find each other with a warp match -- and scatters them.
+// 4-bit digits (16 passes, counts in registers) took 0.43 ms at 2^18 keys.
 // ---------------------------------------------------------------------------
 
 __global__ void __launch_bounds__(kSortNT) sort_hist_kernel(int64_t n, const uint64_t *__restrict__ key,
@@ -211,50 +234,63 @@ __global__ void __launch_bounds__(kSortNT) sort_hist_kernel(int64_t n, const uin
                                                             int64_t nb)
 {
     __shared__ int32_t cnt[kBins];
-    if (threadIdx.x < kBins) cnt[threadIdx.x] = 0;
+    cnt[threadIdx.x] = 0;
     __syncthreads();
-    const int64_t base = (int64_t)blockIdx.x * kSortBlock + (int64_t)threadIdx.x * kSortPer;
-    int32_t local[kBins];
-#pragma unroll
-    for (int d = 0; d < kBins; ++d) local[d] = 0;
+    const int64_t base = (int64_t)blockIdx.x * kSortBlock;
 #pragma unroll
     for (int k = 0; k < kSortPer; ++k) {
-        const int64_t s = base + k;
-        if (s < n) {
-            const int d = (int)((key[s] >> shift) & 15u);
-#pragma unroll
-            for (int e = 0; e < kBins; ++e) local[e] += (d == e);
-        }
+        const int64_t s = base + k * kSortNT + threadIdx.x;
+        if (s < n) atomicAdd(&cnt[(key[s] >> shift) & (kBins - 1)], 1);
     }
-#pragma unroll
-    for (int d = 0; d < kBins; ++d)
-        if (local[d]) atomicAdd(&cnt[d], local[d]);
     __syncthreads();
-    if (threadIdx.x < kBins) hist[(int64_t)threadIdx.x * nb + blockIdx.x] = cnt[threadIdx.x];
+    hist[(int64_t)threadIdx.x * nb + blockIdx.x] = cnt[threadIdx.x];
 }
+static_assert(kSortNT == kBins, "one thread per digit");
 
 // Exclusive scan, in place, of hist[0 .. total) (digit-major), one CTA of 1024.
 __global__ void __launch_bounds__(1024) sort_scan_kernel(int32_t *__restrict__ hist, int64_t total)
 {
-    __shared__ int32_t part[1024];
-    const int64_t per = (total + 1023) / 1024;
-    const int64_t a = threadIdx.x * per;
-    const int64_t b = a + per < total ? a + per : total;
-    int32_t s = 0;
-    for (int64_t k = a; k < b; ++k) s += hist[k];
-    part[threadIdx.x] = s;
+    __shared__ int32_t wsum[32];
+    __shared__ int32_t carry;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    if (threadIdx.x == 0) carry = 0;
     __syncthreads();
-    for (int o = 1; o < 1024; o <<= 1) {
-        const int32_t v = threadIdx.x >= o ? part[threadIdx.x - o] : 0;
+    for (int64_t b0 = 0; b0 < total; b0 += 4096) {
+        const int64_t at = b0 + 4 * (int64_t)threadIdx.x;
+        int32_t v[4];
+        int32_t s = 0;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            v[q] = at + q < total ? hist[at + q] : 0;
+            s += v[q];
+        }
+        int32_t x = s;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int32_t y = __shfl_up_sync(0xffffffffu, x, o);
+            if (lane >= o) x += y;
+        }
+        if (lane == 31) wsum[wid] = x;
         __syncthreads();
-        part[threadIdx.x] += v;
+        if (wid == 0) {
+            int32_t t = wsum[lane];
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int32_t y = __shfl_up_sync(0xffffffffu, t, o);
+                if (lane >= o) t += y;
+            }
+            wsum[lane] = t;
+        }
         __syncthreads();
-    }
-    int32_t run = part[threadIdx.x] - s;
-    for (int64_t k = a; k < b; ++k) {
-        const int32_t v = hist[k];
-        hist[k] = run;
-        run += v;
+        int32_t run = carry + (wid ? wsum[wid - 1] : 0) + x - s;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            if (at + q < total) hist[at + q] = run;
+            run += v[q];
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) carry += wsum[31];
+        __syncthreads();
     }
 }
 
@@ -263,45 +299,43 @@ __global__ void __launch_bounds__(kSortNT) sort_scatter_kernel(
     uint64_t *__restrict__ key_out, int32_t *__restrict__ val_out, int shift,
     const int32_t *__restrict__ hist, int64_t nb)
 {
-    __shared__ int32_t cnt[kBins][kSortNT + 1];
-    const int64_t base = (int64_t)blockIdx.x * kSortBlock + (int64_t)threadIdx.x * kSortPer;
-    int32_t local[kBins];
-#pragma unroll
-    for (int d = 0; d < kBins; ++d) local[d] = 0;
+    __shared__ int32_t cnt[kSortWarps][kBins];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    for (int w = 0; w < kSortWarps; ++w) cnt[w][threadIdx.x] = 0;
+    __syncthreads();
+    const int64_t base = (int64_t)blockIdx.x * kSortBlock + (int64_t)wid * (32 * kSortPer) + lane;
+    uint64_t kk[kSortPer];
+    int32_t rank[kSortPer];            // among the warp's earlier keys of the digit
 #pragma unroll
     for (int k = 0; k < kSortPer; ++k) {
-        const int64_t s = base + k;
-        if (s < n) {
-            const int d = (int)((key_in[s] >> shift) & 15u);
-#pragma unroll
-            for (int e = 0; e < kBins; ++e) local[e] += (d == e);
-        }
+        const int64_t s = base + 32 * k;
+        const bool real = s < n;
+        kk[k] = real ? key_in[s] : 0;
+        // (places past the end: a digit of their own)
+        const uint32_t d = real ? (uint32_t)(kk[k] >> shift) & (kBins - 1) : kBins;
+        const uint32_t same = __match_any_sync(0xffffffffu, d);
+        const int before = real ? cnt[wid][d] : 0;
+        rank[k] = before + __popc(same & ((1u << lane) - 1u));
+        __syncwarp();
+        if (real && lane == 31 - __clz(same)) cnt[wid][d] = before + __popc(same);
+        __syncwarp();
     }
-#pragma unroll
-    for (int d = 0; d < kBins; ++d) cnt[d][threadIdx.x] = local[d];
     __syncthreads();
-    if (threadIdx.x < kBins) {                 // exclusive scan over the threads, per digit
+    {   // per digit: this CTA's first place, then each warp's
         int32_t run = hist[(int64_t)threadIdx.x * nb + blockIdx.x];
-        for (int t = 0; t < kSortNT; ++t) {
-            const int32_t v = cnt[threadIdx.x][t];
-            cnt[threadIdx.x][t] = run;
+        for (int w = 0; w < kSortWarps; ++w) {
+            const int32_t v = cnt[w][threadIdx.x];
+            cnt[w][threadIdx.x] = run;
             run += v;
         }
     }
     __syncthreads();
 #pragma unroll
-    for (int d = 0; d < kBins; ++d) local[d] = cnt[d][threadIdx.x];
-#pragma unroll
     for (int k = 0; k < kSortPer; ++k) {
-        const int64_t s = base + k;
+        const int64_t s = base + 32 * k;
         if (s < n) {
-            const uint64_t kk = key_in[s];
-            const int d = (int)((kk >> shift) & 15u);
-            int32_t at = 0;
-#pragma unroll
-            for (int e = 0; e < kBins; ++e)
-                if (d == e) at = local[e]++;
-            key_out[at] = kk;
+            const int32_t at = cnt[wid][(kk[k] >> shift) & (kBins - 1)] + rank[k];
+            key_out[at] = kk[k];
             val_out[at] = val_in[s];
         }
     }
@@ -313,10 +347,9 @@ __global__ void __launch_bounds__(kSortNT) sort_scatter_kernel(
 
 __global__ void tree_init_kernel(TreeView t)
 {
+    if (threadIdx.x < 24) t.counters[32 + threadIdx.x] = threadIdx.x == 0;   // nodes per level
     if (threadIdx.x != 0) return;
-    t.counters[0] = 1;
     t.counters[1] = 0;   // level 0 starts at node 0
-    t.counters[2] = 1;   // level 1 starts at node 1
     t.first[0] = 0;
     t.count[0] = (int32_t)t.n;
     t.level[0] = 0;
@@ -339,9 +372,19 @@ __device__ __forceinline__ int32_t digit_bound(const uint64_t *key, int32_t a, i
     return a;
 }
 
+// Splits the nodes of level lvl.  The level's range follows from the counts of
+// the levels above; the children of all its nodes are appended behind it, each
+// linked to its next sibling or, the last, to its parent's next.
 __global__ void __launch_bounds__(256) tree_split_kernel(TreeView t, int lvl)
 {
-    const int32_t lb = t.counters[1 + lvl], le = t.counters[2 + lvl];
+    const int32_t lb = t.counters[1 + lvl];
+    int64_t end = (int64_t)lb + t.counters[32 + lvl];
+    if (end > t.max_nodes) end = t.max_nodes;
+    const int32_t le = (int32_t)end;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        t.counters[2 + lvl] = le;                    // first node of the next level
+        if (lvl == kMaxLevel) t.counters[0] = le;    // all nodes
+    }
     for (int32_t k = lb + (int32_t)(blockIdx.x * 256 + threadIdx.x); k < le;
          k += (int32_t)(gridDim.x * 256)) {
         t.child_first[k] = -1;
@@ -355,32 +398,25 @@ __global__ void __launch_bounds__(256) tree_split_kernel(TreeView t, int lvl)
         for (uint32_t o = 1; o < 8; ++o) edge[o] = digit_bound(t.key, edge[o - 1], f + c, shift, o);
         int nc = 0;
         for (int o = 0; o < 8; ++o) nc += edge[o + 1] > edge[o];
-        const int32_t base = atomicAdd(&t.counters[0], nc);
-        if ((int64_t)base + nc > t.max_nodes) {
+        const int64_t base = (int64_t)le + atomicAdd(&t.counters[33 + lvl], nc);
+        if (base + nc > t.max_nodes) {
             flag_or(t.flags, GRAV_FLAG_OVERFLOW);
             continue;
         }
+        const int32_t up = t.next[k];
         int q = 0;
         for (int o = 0; o < 8; ++o) {
             if (edge[o + 1] == edge[o]) continue;
-            const int32_t ch = base + q++;
+            const int32_t ch = (int32_t)base + q++;
             t.first[ch] = edge[o];
             t.count[ch] = edge[o + 1] - edge[o];
             t.level[ch] = (int8_t)(lvl + 1);
             t.child_first[ch] = -1;
             t.n_child[ch] = 0;
+            t.next[ch] = q < nc ? ch + 1 : up;
         }
-        t.child_first[k] = base;
+        t.child_first[k] = (int32_t)base;
         t.n_child[k] = (int8_t)nc;
-    }
-}
-
-__global__ void tree_mark_kernel(TreeView t, int lvl)
-{
-    if (threadIdx.x == 0) {
-        int64_t n = t.counters[0];
-        if (n > t.max_nodes) n = t.max_nodes;
-        t.counters[3 + lvl] = (int32_t)n;   // first node of level lvl + 2
     }
 }
 
@@ -421,17 +457,6 @@ __global__ void __launch_bounds__(256) tree_moment_kernel(TreeView t, const doub
             t.com[3 * (int64_t)k + e] = m > 0.0 ? __ddiv_rn(mx[e], m) : 0.0;
             t.vcom[3 * (int64_t)k + e] = m > 0.0 ? __ddiv_rn(mv[e], m) : 0.0;
         }
-    }
-}
-
-__global__ void __launch_bounds__(256) tree_next_kernel(TreeView t, int lvl)
-{
-    const int32_t lb = t.counters[1 + lvl], le = t.counters[2 + lvl];
-    for (int32_t k = lb + (int32_t)(blockIdx.x * 256 + threadIdx.x); k < le;
-         k += (int32_t)(gridDim.x * 256)) {
-        const int32_t cf = t.child_first[k];
-        const int nc = t.n_child[k];
-        for (int q = 0; q < nc; ++q) t.next[cf + q] = (q + 1 < nc) ? cf + q + 1 : t.next[k];
     }
 }
 
@@ -867,9 +892,9 @@ extern "C" int grav_eval_tree(const grav_params *p, const grav_tree_params *tp, 
 
     // bounding cube and keys
     const int nbb = (int)std::min<int64_t>(kBboxBlocks, (n + 255) / 256);
-    double *part = reinterpret_cast<double *>(ws + L.part);
+    long long *part = reinterpret_cast<long long *>(ws + L.part);
     bbox_partial_kernel<<<nbb, 256, 0, st>>>(n, pos, part);
-    bbox_final_kernel<<<1, 32, 0, st>>>(nbb, part, t.frame);
+    bbox_final_kernel<<<1, 256, 0, st>>>(nbb, part, t.frame);
     uint64_t *ka = reinterpret_cast<uint64_t *>(ws + L.key_a), *kb = reinterpret_cast<uint64_t *>(ws + L.key_b);
     int32_t *va = reinterpret_cast<int32_t *>(ws + L.val_a), *vb = reinterpret_cast<int32_t *>(ws + L.val_b);
     key_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(n, pos, t.frame, ka, va, flags_dev);
@@ -880,7 +905,7 @@ extern "C" int grav_eval_tree(const grav_params *p, const grav_tree_params *tp, 
     int32_t *hist = reinterpret_cast<int32_t *>(ws + L.hist);
     const int64_t nb = L.n_sort_blocks;
     for (int pass = 0; pass < kPasses; ++pass) {
-        const int shift = 4 * pass;
+        const int shift = 8 * pass;
         sort_hist_kernel<<<(unsigned)nb, kSortNT, 0, st>>>(n, ka, shift, hist, nb);
         sort_scan_kernel<<<1, 1024, 0, st>>>(hist, nb * kBins);
         sort_scatter_kernel<<<(unsigned)nb, kSortNT, 0, st>>>(n, ka, va, kb, vb, shift, hist, nb);
@@ -892,18 +917,20 @@ extern "C" int grav_eval_tree(const grav_params *p, const grav_tree_params *tp, 
     t.key = ka;
     t.order = va;
 
-    // levels: split top-down, moments bottom-up, next links top-down
-    const unsigned g = (unsigned)std::min<int64_t>(4096, (L.max_nodes + 255) / 256);
+    // levels: split and link top-down, moments bottom-up.  Most of the 22
+    // levels are empty or small: a grid of a few CTAs per SM strides over the
+    // full ones (grids of 4096 CTAs took 5 us for an empty level)
+    int sms = 0;
+    rc = device_sm_count(&sms);
+    if (rc) return rc;
+    const unsigned g = (unsigned)std::min<int64_t>(4LL * sms, (L.max_nodes + 255) / 256);
     tree_init_kernel<<<1, 32, 0, st>>>(t);
-    for (int lvl = 0; lvl <= kMaxLevel; ++lvl) {
-        tree_split_kernel<<<g, 256, 0, st>>>(t, lvl);
-        tree_mark_kernel<<<1, 32, 0, st>>>(t, lvl);
-    }
+    for (int lvl = 0; lvl <= kMaxLevel; ++lvl) tree_split_kernel<<<g, 256, 0, st>>>(t, lvl);
     for (int lvl = kMaxLevel; lvl >= 0; --lvl)
         tree_moment_kernel<<<g, 256, 0, st>>>(t, pos, vel, mass, lvl);
-    for (int lvl = 0; lvl < kMaxLevel; ++lvl) tree_next_kernel<<<g, 256, 0, st>>>(t, lvl);
     const bool mixed = p->precision == GRAV_MIXED;
-    tree_walk_data_kernel<<<g, 256, 0, st>>>(t, pos, vel, mass, mixed);
+    tree_walk_data_kernel<<<(unsigned)std::min<int64_t>(4096, (L.max_nodes + 255) / 256), 256, 0, st>>>(
+        t, pos, vel, mass, mixed);
     rc = check_launch("grav_eval_tree/build");
     if (rc) return rc;
     if (order_out) {
