@@ -20,7 +20,7 @@
 // own element is farther than its radius from the box, and otherwise
 // pre-filters every source with an FP32 distance test that carries an explicit
 // bound on its rounding.  What passes is listed, with its FP64 distance, up to
-// 1.25 times the support, and the Newton passes run over the lists: a scan is
+// 1.2 times the support, and the Newton passes run over the lists: a scan is
 // repeated only for supports that outgrow their list.  In each pass a thread
 // first collects the listed sources inside its support (integer compares of
 // the FP64 bits), then sums W, dW/dh and dpsi/dh over them, so the lanes of a
@@ -192,8 +192,8 @@ __device__ __forceinline__ bool box_near(const float blo[3], const float bhi[3],
     return d2 < __fmul_ru(H, H);
 }
 
-constexpr int kSoftList = 224;      // listed sources per element
-constexpr double kSoftReach = 1.25; // list radius over the support it is made for
+constexpr int kSoftList = 144;      // listed sources per element (local memory)
+constexpr double kSoftReach = 1.2;  // list radius over the support it is made for
 
 __global__ void __launch_bounds__(kSoftNT) soft_solve_kernel(SoftArgs a)
 {
@@ -221,23 +221,23 @@ __global__ void __launch_bounds__(kSoftNT) soft_solve_kernel(SoftArgs a)
     int32_t it = 0;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const float inf = __int_as_float(0x7f800000);
-    // the list: sources within `reach` in ascending order, and their FP64
-    // squared distances and distances
+    // the list: sources within `reach` in ascending order and their distances
     int32_t nj[kSoftList];
-    double nr2[kSoftList], nr[kSoftList];
+    double nr[kSoftList];
     int cnt = 0;
     double reach = 0.0;
-    bool direct = false;      // more sources in reach than the list holds
 
     for (int pass = 0; pass < a.max_iter; ++pass) {
         if (!__syncthreads_or(!done)) break;       // every element of the CTA is done
         double rho = 0.0, rho_h = 0.0, psi_h = 0.0;
         const double hinv = 1.0 / h, h2 = h * h;
-        // ---- scans: lists for the supports that outgrew theirs, the sums of
-        // the elements without a list (a second scan when a list overflows)
-        bool want = !done && (direct || h > reach);
+        // ---- scans: lists for the supports that outgrew theirs; one that
+        // overflows is made for the support alone in a second scan, and when
+        // that overflows too a third scan sums the element directly
+        bool want = !done && h > reach, direct = false;
+        double factor = kSoftReach;
         while (__syncthreads_or(want)) {
-            const double rad = direct ? h : kSoftReach * h;
+            const double rad = factor * h;
             float l[3], u[3], hm = want ? __double2float_ru(rad) : 0.0f;
             for (int c = 0; c < 3; ++c) {
                 l[c] = want ? __double2float_rd(xi[c]) : inf;
@@ -345,18 +345,15 @@ __global__ void __launch_bounds__(kSoftNT) soft_solve_kernel(SoftArgs a)
             }
             if (want) {
                 if (!direct && cnt > kSoftList) {
-                    direct = true;                 // sum this pass in another scan
+                    direct = factor == 1.0;
+                    factor = 1.0;
                 } else {
                     want = false;
-                    if (!direct) {
-                        reach = rad;
-                        for (int k = 0; k < cnt; ++k) {
-                            const double4 s = a.src[nj[k]];
-                            const double dx = s.x - xi[0], dy = s.y - xi[1], dz = s.z - xi[2];
-                            const double r2 = fma(dx, dx, fma(dy, dy, dz * dz));
-                            nr2[k] = r2;
-                            nr[k] = sqrt(r2);
-                        }
+                    reach = direct ? 0.0 : rad;
+                    for (int k = 0; k < (direct ? 0 : cnt); ++k) {
+                        const double4 s = a.src[nj[k]];
+                        const double dx = s.x - xi[0], dy = s.y - xi[1], dz = s.z - xi[2];
+                        nr[k] = sqrt(fma(dx, dx, fma(dy, dy, dz * dz)));
                     }
                 }
             }
@@ -364,11 +361,13 @@ __global__ void __launch_bounds__(kSoftNT) soft_solve_kernel(SoftArgs a)
 
         // ---- sums over the listed sources inside the support ----
         if (!done && !direct) {
+            // (r < h where the scan asks r^2 < h^2: the two differ at most where
+            // r / h rounds to 1, where every term is zero)
             uint8_t in[kSoftList];
             int n_in = 0;
-            const long long h2b = __double_as_longlong(h2);      // (non-negative: ordered as integers)
+            const long long hb = __double_as_longlong(h);        // (non-negative: ordered as integers)
             for (int k = 0; k < cnt; ++k)
-                if (__double_as_longlong(nr2[k]) < h2b) in[n_in++] = (uint8_t)k;
+                if (__double_as_longlong(nr[k]) < hb) in[n_in++] = (uint8_t)k;
             for (int q = 0; q < n_in; ++q) {
                 const int k = in[q];
                 const int32_t j = nj[k];
