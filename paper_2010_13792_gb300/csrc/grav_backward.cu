@@ -156,19 +156,15 @@ __device__ __forceinline__ void bwd_df_loop(const float4 *__restrict__ P, const 
     }
 }
 
-// One pair of the adjoint in FP64 (d, a_bar given): added to s[kNB].  The
-// Newtonian powers are corrected for the rounding of rsqrt as in the forward.
+// One pair of the adjoint in FP64 (d, a_bar given): added to s[kNB].
 __device__ __forceinline__ void bwd_pair_fp64(const double d[3], const double ab[3], double h2, double hinv,
                                               double hinv3, double hinv5, bool self, double s[kNB])
 {
     const double r2 = fma(d[0], d[0], fma(d[1], d[1], d[2] * d[2]));
     const double ri = rsqrt(r2);
     const double ri2 = ri * ri;
-    const double t = fma(-r2, fma(ri, ri, -ri2), fma(-r2, ri2, 1.0));
     double f = ri * ri2;
-    f = fma(f, 1.5 * t, f);
     double gp = f * ri2;
-    gp = fma(gp, t, gp);
     if (r2 < h2) {
         double F, Gp, P;
         spline_kernel<double>(sqrt(r2) * hinv, F, Gp, P);

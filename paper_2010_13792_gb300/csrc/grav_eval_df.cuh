@@ -121,22 +121,26 @@ __device__ __forceinline__ void df_sub_loop(const float4 *__restrict__ P, const 
     }
 }
 
-// One pair in FP64: the Newtonian inverse powers are corrected for the
-// rounding of rsqrt (t = 1 - r^2 y^2, as in the two-part loop), since these few
-// pairs carry most of a target's rounding; the cubic spline inside h.
-template <bool POT>
+// One pair in FP64, the cubic spline inside h.  LISTED: the Newtonian inverse
+// powers are corrected for the rounding of rsqrt (t = 1 - r^2 y^2, as in the
+// two-part loop), since these few pairs carry most of a target's rounding.
+template <bool POT, bool LISTED>
 __device__ __forceinline__ void df_pair_terms(double r2, double m, double h2, double hinv, double hinv3,
                                               double hinv5, double &mf, double &mg, double &mp)
 {
     const double ri = rsqrt(r2);
     const double ri2 = ri * ri;
-    const double t = fma(-r2, fma(ri, ri, -ri2), fma(-r2, ri2, 1.0));
     mp = m * ri;
     mf = mp * ri2;
-    mf = fma(mf, 1.5 * t, mf);
-    mg = mf * ri2;
-    mg = fma(mg, t, mg);
-    if (POT) mp = fma(mp, 0.5 * t, mp);
+    if (LISTED) {
+        const double t = fma(-r2, fma(ri, ri, -ri2), fma(-r2, ri2, 1.0));
+        mf = fma(mf, 1.5 * t, mf);
+        mg = mf * ri2;
+        mg = fma(mg, t, mg);
+        if (POT) mp = fma(mp, 0.5 * t, mp);
+    } else {
+        mg = mf * ri2;
+    }
     if (r2 < h2) {
         double F, Gp, P;
         spline_kernel<double>(sqrt(r2) * hinv, F, Gp, P);
@@ -163,7 +167,7 @@ __device__ __noinline__ void df_flush(const double *__restrict__ pos, const doub
         const int64_t j = list[k];
         const double dx = pos[3 * j] - xi[0], dy = pos[3 * j + 1] - xi[1], dz = pos[3 * j + 2] - xi[2];
         double mf, mg, mp;
-        df_pair_terms<POT>(fma(dx, dx, fma(dy, dy, dz * dz)), mass[j], h2, hinv, hinv3, hinv5, mf, mg, mp);
+        df_pair_terms<POT, true>(fma(dx, dx, fma(dy, dy, dz * dz)), mass[j], h2, hinv, hinv3, hinv5, mf, mg, mp);
         accumulate_d<POT>(acc, dx, dy, dz, vel[3 * j] - vi[0], vel[3 * j + 1] - vi[1],
                           vel[3 * j + 2] - vi[2], mf, mg, mp);
     }
@@ -192,7 +196,8 @@ __device__ __forceinline__ void df_fp64_loop(const EvalArgs &a, const TileGeom &
         const int64_t j = first + k;
         const double dx = a.pos[3 * j] - xi[0], dy = a.pos[3 * j + 1] - xi[1], dz = a.pos[3 * j + 2] - xi[2];
         double mf, mg, mp;
-        df_pair_terms<POT>(fma(dx, dx, fma(dy, dy, dz * dz)), a.mass[j], h2, hinv, hinv3, hinv5, mf, mg, mp);
+        df_pair_terms<POT, false>(fma(dx, dx, fma(dy, dy, dz * dz)), a.mass[j], h2, hinv, hinv3, hinv5, mf, mg,
+                                  mp);
         if (j == ti) {
             mf = 0.0;
             mg = 0.0;
