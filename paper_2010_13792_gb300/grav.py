@@ -153,6 +153,8 @@ def lib_path() -> str:
 def lib():
     """The loaded libgrav handle.  Raises if the library has not been built."""
     global _lib
+    if _lib is not None:        # set once, under the lock
+        return _lib
     with _lock:
         if _lib is not None:
             return _lib
@@ -177,16 +179,23 @@ def _err(where: str, rc: int):
 
 
 def _stream(stream=None):
+    """The cudaStream_t (an int, as ctypes takes it for a void pointer)."""
     if stream is None:
         stream = torch.cuda.current_stream()
-    return ctypes.c_void_p(stream.cuda_stream)
+    return stream.cuda_stream
 
 
 def _ptr(t, dtype, name, shape=None, allow_none=False):
+    """The device address of a checked tensor (an int; 0 if it has no elements).
+    A call checks up to a dozen tensors: the tests run in one expression, and
+    which of them failed is looked up only then."""
     if t is None:
         if allow_none:
             return None
         raise GravError(GRAV_EINVAL, name, "tensor required")
+    if (isinstance(t, torch.Tensor) and t.dtype is dtype and t.is_cuda and t.is_contiguous()
+            and (shape is None or t.shape == shape)):
+        return t.data_ptr()
     if not isinstance(t, torch.Tensor):
         raise GravError(GRAV_EINVAL, name, "expected a torch.Tensor")
     if not t.is_cuda:
@@ -197,7 +206,7 @@ def _ptr(t, dtype, name, shape=None, allow_none=False):
         raise GravError(GRAV_EINVAL, name, "tensor must be contiguous")
     if shape is not None and tuple(t.shape) != tuple(shape):
         raise GravError(GRAV_EINVAL, name, f"shape {tuple(t.shape)}, expected {tuple(shape)}")
-    return ctypes.c_void_p(t.data_ptr()) if t.numel() else ctypes.c_void_p(0)
+    return t.data_ptr()
 
 
 def version() -> str:
@@ -285,7 +294,7 @@ def compact_active(flags_u8, idx_out, count_out, workspace: Workspace | None = N
     buf = _ws(workspace, "compact", dev).get(nb, dev)
     rc = lib().grav_compact_active(
         n, _ptr(flags_u8, torch.uint8, "flags", (n,)), _ptr(idx_out, torch.int32, "idx_out", (n,)),
-        _ptr(count_out, torch.int32, "count_out", (1,)), ctypes.c_void_p(buf.data_ptr()), nb,
+        _ptr(count_out, torch.int32, "count_out", (1,)), buf.data_ptr(), nb,
         _stream(stream))
     _err("grav_compact_active", rc)
 
@@ -375,7 +384,7 @@ def eval_active(p: Params, pos, vel, mass, idx, n_idx_dev, n_idx_max: int, acc, 
         _ptr(pot, torch.float64, "pot", (n,), allow_none=True),
         _ptr(dt_grav, torch.float64, "dt_grav", (n,), allow_none=True),
         _ptr(flags, torch.int32, "flags", (1,), allow_none=True),
-        ctypes.c_void_p(buf.data_ptr()), nb, _stream(stream))
+        buf.data_ptr(), nb, _stream(stream))
     _err("grav_eval_active", rc)
 
 
@@ -400,7 +409,7 @@ def soft_solve(sp: SoftParams, pos, mass, h, zeta=None, omega=None, iters=None, 
         _ptr(omega, torch.float64, "omega", (n,), allow_none=True),
         _ptr(iters, torch.int32, "iters", (n,), allow_none=True),
         _ptr(flags, torch.int32, "flags", (1,), allow_none=True),
-        ctypes.c_void_p(buf.data_ptr()), nb, _stream(stream))
+        buf.data_ptr(), nb, _stream(stream))
     _err("grav_soft_solve", rc)
 
 
@@ -429,7 +438,7 @@ def eval_soft(p: Params, pos, vel, mass, h, zeta, idx, n_idx_dev, n_idx_max: int
         _ptr(pot, torch.float64, "pot", (n,), allow_none=True),
         _ptr(dt_grav, torch.float64, "dt_grav", (n,), allow_none=True),
         _ptr(flags, torch.int32, "flags", (1,), allow_none=True),
-        ctypes.c_void_p(buf.data_ptr()), nb, _stream(stream))
+        buf.data_ptr(), nb, _stream(stream))
     _err("grav_eval_soft", rc)
 
 
@@ -461,7 +470,7 @@ def eval_tree(p: Params, tp: TreeParams, pos, vel, mass, idx, n_idx_dev, n_idx_m
         _ptr(order, torch.int32, "order", (n,), allow_none=True),
         _ptr(stats, torch.int64, "stats", (2,), allow_none=True),
         _ptr(flags, torch.int32, "flags", (1,), allow_none=True),
-        ctypes.c_void_p(buf.data_ptr()), nb, _stream(stream))
+        buf.data_ptr(), nb, _stream(stream))
     _err("grav_eval_tree", rc)
 
 
@@ -517,7 +526,7 @@ def eval_batched(p: Params, systems, pos, vel, mass, idx, n_idx_dev, n_idx_max: 
         _ptr(pot, torch.float64, "pot", (n,), allow_none=True),
         _ptr(dt_grav, torch.float64, "dt_grav", (n,), allow_none=True),
         _ptr(flags, torch.int32, "flags", (1,), allow_none=True),
-        ctypes.c_void_p(buf.data_ptr()), nb, _stream(stream))
+        buf.data_ptr(), nb, _stream(stream))
     _err("grav_eval_batched", rc)
 
 
@@ -544,7 +553,7 @@ def eval_backward(p: Params, pos, mass, a_bar, w_bar: float, acc, tidal, pot, po
         _ptr(pos_bar, torch.float64, "pos_bar", (n, 3)),
         _ptr(mass_bar, torch.float64, "mass_bar", (n,)),
         _ptr(flags, torch.int32, "flags", (1,), allow_none=True),
-        ctypes.c_void_p(buf.data_ptr()), nb, _stream(stream))
+        buf.data_ptr(), nb, _stream(stream))
     _err("grav_eval_backward", rc)
 
 
@@ -575,7 +584,7 @@ def eval_backward_batched(p: Params, systems, pos, mass, a_bar, w_bar: float, ac
         _ptr(pos_bar, torch.float64, "pos_bar", (n, 3)),
         _ptr(mass_bar, torch.float64, "mass_bar", (n,)),
         _ptr(flags, torch.int32, "flags", (1,), allow_none=True),
-        ctypes.c_void_p(buf.data_ptr()), nb, _stream(stream))
+        buf.data_ptr(), nb, _stream(stream))
     _err("grav_eval_backward_batched", rc)
 
 
