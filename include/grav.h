@@ -113,7 +113,9 @@ GRAV_API int grav_tile_config(int32_t precision, int32_t index, grav_tile_info *
  * n_targets targets (the n_idx_max of the call): open boundaries
  * (periodic = soft = 0), a periodic box (periodic != 0) or adaptive softening
  * (soft != 0).  768-thread CTAs from 8192 targets, 256-thread CTAs below
- * (the same in every mode).  Returns
+ * (the same in every mode).  Below 2^30 interactions (targets x sources) an
+ * open-boundary evaluation then takes 128-thread CTAs on the same tiles, by the count on the
+ * device where it is there.  Returns
  * the index (>= 0), or GRAV_EINVAL for a bad precision or n_targets < 0.  A
  * property of the library's kernels; the paper has no counterpart. */
 GRAV_API int32_t grav_default_tile_config(int32_t precision, int32_t periodic, int32_t soft,

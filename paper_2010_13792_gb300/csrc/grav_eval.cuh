@@ -114,6 +114,13 @@ struct EvalArgs {
     const double *zeta;
     const float2 *hz;
     const float *geo_h;
+
+    // two launches share one evaluation whose count is on the device: the
+    // kernel of few targets runs below `few` targets (few > 0), the other
+    // from -few targets on (few < 0); 0: a single launch.  The reduction takes
+    // the block size and grid of the one that ran.
+    int64_t few;
+    int32_t few_grid, few_bt;
 };
 
 // Number of source chunks per target block.  Shared by the host, the eval
@@ -2323,6 +2330,7 @@ eval_mixed_kernel(const EvalArgs a)
     init_mixed_ring(sm);
     Ring ring{0u, 0u};
     const int64_t n_act = active_count(a);
+    if (a.few > 0 ? n_act >= a.few : n_act < -a.few) return;      // the other launch's evaluation
     const int64_t n_tb = (n_act + BT - 1) / BT;
     const int split = choose_split(n_tb, a.n_tiles, a.grid, a.max_split, a.part_cap_rows, BT);
     const int64_t items = n_tb * split;
@@ -2666,8 +2674,10 @@ reduce_partials_kernel(const EvalArgs a, int32_t BT)
     constexpr int TPB = reduce_targets_per_block<POT>();
     __shared__ double red[NC][TPB];
     const int64_t n_act = active_count(a);
+    const bool few = n_act < -a.few;
+    if (few) BT = a.few_bt;
     const int64_t n_tb = (n_act + BT - 1) / BT;
-    const int split = choose_split(n_tb, a.n_tiles, a.grid, a.max_split, a.part_cap_rows, BT);
+    const int split = choose_split(n_tb, a.n_tiles, few ? a.few_grid : a.grid, a.max_split, a.part_cap_rows, BT);
     if (split <= 1) return;
     const int64_t rows = n_tb * BT;
     const int k = threadIdx.x % TPB, c = threadIdx.x / TPB;
