@@ -226,7 +226,9 @@ class Path:
         self.params = grav.params(h=H, precision=grav.MIXED, tile_config=tile_config)
         self.ws_compact = grav.Workspace()
         self.ws_eval = grav.Workspace()
-        self.launches_per_step = 9   # select 1, compact 3, pack 1, eval 1, reduce 1, predict 1, bins 1
+        # select 1, compact 3, pack 1, eval 1 (2 with the default configuration: the count
+        # on the device decides which works), reduce 1, predict 1, bins 1
+        self.launches_per_step = 9 if tile_config >= 0 else 10
 
     def step(self, tick, ev=None):
         """One pass of the path at `tick` (odd ticks: only the fine bin is active)."""

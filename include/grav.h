@@ -304,8 +304,8 @@ GRAV_API int grav_eval_backward(const grav_params *p, int64_t n, const double *p
  * DEVICE array of grav_eval_batched ({offset, n, h}, h = 0: p->h); every
  * element of a system is a target, and its sums run over its own system's
  * elements only, with its system's support h.  Work items are (system,
- * target block) pairs taken longest system first through an atomic ticket;
- * each element's sums are formed by one CTA over its system's tiles in a
+ * target block) pairs, longest system first, dealt to one queue per SM with
+ * stealing; each element's sums are formed by one CTA over its system's tiles in a
  * fixed order, so a system's results equal grav_eval_backward on that system
  * alone with max_split = 1, bit for bit.  Elements of no system, and of a
  * system that is skipped (out of range, overlapping, bad h: see
@@ -338,8 +338,9 @@ GRAV_API int grav_eval_backward_batched(const grav_params *p, int32_t n_sys, con
  * the call can be captured in a CUDA graph.  Outputs are scattered to the
  * targets' rows as in grav_eval_active.
  * Work is split into (system, target block) items, ordered by decreasing
- * per-item cost (system size) and taken by a fixed grid of CTAs through an
- * atomic ticket; each target's sum is formed by one CTA over its system's
+ * per-item cost (system size), dealt to one queue per SM and taken by a fixed
+ * grid of CTAs, which steal from other queues once theirs is empty; each
+ * target's sum is formed by one CTA over its system's
  * tiles in a fixed order, so results do not depend on scheduling and equal
  * grav_eval_active on that system alone with max_split = 1.
  * A system that is out of range, overlaps its predecessor or has an h that

@@ -180,11 +180,6 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t *bar, uint32_t parity
     return false;
 }
 
-__device__ __forceinline__ bool finite3(double a, double b, double c)
-{
-    return isfinite(a) && isfinite(b) && isfinite(c);
-}
-
 // Tidal timestep, Eq. (tidaltimestep): sqrt(eta) * (||T||_F^2 / 6)^(-1/4),
 // ||T||^2 summed in the fixed order xx, yy, zz, then 2xy^2, 2xz^2, 2yz^2,
 // every operation correctly rounded (no contraction); +inf for T = 0.

@@ -27,7 +27,7 @@
 // warp run the FP64 terms side by side: FP64 bounds this kernel, and with the
 // terms inside the scan a warp ran them once for every source inside any of
 // its 32 supports, 12 lanes active (40961 elements, n_ngb = 32, guesses off by
-// up to 20%: 8.1 ms, with the lists 4.1 ms).  An element with more than
+// up to 20%: 8.1 ms, with the lists 3.0 ms).  An element with more than
 // kSoftList sources in reach sums them in the scans.  Every order of summation
 // is that of the sources.  Newton steps are limited to a factor of 2 in h.
 // Every loop is bounded by max_iter passes.
