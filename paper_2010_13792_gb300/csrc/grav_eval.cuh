@@ -2482,8 +2482,9 @@ eval_mixed_batched_kernel(const EvalArgs a, const BatchView b)
 }
 
 // ---------------------------------------------------------------------------
-// K4: FP64 force kernel of the periodic box and of adaptive softening (one
-// target per thread; open boundaries: grav_eval_df.cuh)
+// K4: FP64 force kernel of the periodic box, of adaptive softening and of the
+// smallest open evaluations (one target per thread; other open boundaries:
+// grav_eval_df.cuh)
 // ---------------------------------------------------------------------------
 
 template <int S>
@@ -2521,10 +2522,14 @@ __device__ __forceinline__ bool f64_item(const EvalArgs &a, F64Smem<S> &sm, Ring
             hi[c] = __double2float_ru(xi[c]);
         }
     }
-    static_assert(MODE != kModeOpen, "open boundaries: df_item (grav_eval_df.cuh)");
     block_bbox<NT>(lo, hi, sm.blo, sm.bhi);
-    const float blo_r[3] = {sm.blo[0], sm.blo[1], sm.blo[2]};
-    const float bhi_r[3] = {sm.bhi[0], sm.bhi[1], sm.bhi[2]};
+    // open boundaries: each warp tests tiles against its own targets' box
+    // (lo/hi now hold it; the near and far loops synchronise nothing)
+    constexpr bool kWarpBox = MODE == kModeOpen;
+    const float blo_r[3] = {kWarpBox ? lo[0] : sm.blo[0], kWarpBox ? lo[1] : sm.blo[1],
+                            kWarpBox ? lo[2] : sm.blo[2]};
+    const float bhi_r[3] = {kWarpBox ? hi[0] : sm.bhi[0], kWarpBox ? hi[1] : sm.bhi[1],
+                            kWarpBox ? hi[2] : sm.bhi[2]};
     // periodic box: the target's close radius (close_radii; the FP64 pair
     // terms need no FP64 close field, only the runs)
     float rc2[1] = {-1.0f};
@@ -2577,9 +2582,11 @@ __device__ __forceinline__ bool f64_item(const EvalArgs &a, F64Smem<S> &sm, Ring
             const int cls = periodic_class<1>(tw, ti1, g, a.h2f_up, a.box_tie_f, rc2);
             close = __syncthreads_or((cls & 2) != 0) != 0;
             near = close || __syncthreads_or((cls & 1) != 0) != 0;
-        } else {
+        } else if (soft) {
             const float hm = fmaxf(h_block, a.geo_h[t]);
             near = tile_is_near(blo_r, bhi_r, g, __fmul_ru(hm, hm));
+        } else {
+            near = tile_is_near(blo_r, bhi_r, g, a.h2f_up);
         }
         const bool got = mbar_wait_bounded(&sm.bar[s], (ring.parity >> s) & 1u, a.flags);
         if (got)
@@ -2617,8 +2624,10 @@ __device__ __forceinline__ bool f64_item(const EvalArgs &a, F64Smem<S> &sm, Ring
             else if (periodic)
                 loop_d<S, POT, true, true>(sm.stage[s], sm.stage[s] + S, xi, i, g.first, h2, hinv,
                                            acc, a.box, a.box_inv, a.box_tie);
-            else
+            else if (!near)
                 loop_d<S, POT, false>(sm.stage[s], sm.stage[s] + S, xi, i, g.first, h2, hinv, acc);
+            else
+                loop_d<S, POT, true>(sm.stage[s], sm.stage[s] + S, xi, i, g.first, h2, hinv, acc);
             target_velocity_d(acc, vr);
         }
 #pragma unroll
@@ -2808,6 +2817,10 @@ struct EvalConfig {
     eval_launch_fn launch_fine[2] = {nullptr, nullptr};
     occupancy_fn occupancy_fine[2] = {nullptr, nullptr};
     pack_launch_fn pack_fine = nullptr;
+    // and in FP64 pair terms
+    eval_launch_fn launch_plain[2] = {nullptr, nullptr};
+    occupancy_fn occupancy_plain[2] = {nullptr, nullptr};
+    pack_launch_fn pack_plain = nullptr;
 };
 
 template <int NT, int KT, int S, int MINB, int U, bool POT, bool SACC, bool PAIR, int MODE>

@@ -58,7 +58,10 @@ int occupancy_df_batched(int *b)
      false,                                                                                        \
      {launch_df<NT, S, false>, launch_df<NT, S, true>},                                            \
      {occupancy_df<NT, S, false>, occupancy_df<NT, S, true>},                                      \
-     launch_pack<S, false, true, false, true>}
+     launch_pack<S, false, true, false, true>,                                                     \
+     {launch_f64<NT, S, false, kModeOpen>, launch_f64<NT, S, true, kModeOpen>},                    \
+     {occupancy_f64<NT, S, false, kModeOpen>, occupancy_f64<NT, S, true, kModeOpen>},              \
+     launch_pack<S, false, true, false>}
 
 static const EvalConfig kF64Configs[] = {
     GRAV_F64_CFG(128, 128),

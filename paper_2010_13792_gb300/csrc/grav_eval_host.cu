@@ -136,11 +136,15 @@ void set_box(EvalArgs &a, double box)
     a.box_lo_f = box > 0.0 ? (float)(box - (double)a.box_f) : 0.0f;
 }
 
-int grid_for(const EvalConfig *c, int index, int mode, bool fine, bool pot, int *grid)
+// Tiles of an evaluation: the configuration's own, and for open FP64 sums the
+// two smaller kinds of tile_kind.
+enum { kNominal = 0, kFine = 1, kPlain = 2 };
+
+int grid_for(const EvalConfig *c, int index, int mode, int tiles, bool pot, int *grid)
 {
     static std::mutex mu;
-    // [device][precision][config][mode, or 3: open on fine tiles][pot]
-    static int cache[64][2][kMaxTileConfigs][4][2];
+    // [device][precision][config][mode, or 3, 4: open on fine or plain tiles][pot]
+    static int cache[64][2][kMaxTileConfigs][5][2];
     int dev = 0;
     int rc = check_cuda(cudaGetDevice(&dev), "cudaGetDevice");
     if (rc) return rc;
@@ -149,10 +153,12 @@ int grid_for(const EvalConfig *c, int index, int mode, bool fine, bool pot, int 
     if (rc) return rc;
     if (dev >= 64 || index >= kMaxTileConfigs) return fail(GRAV_ECUDA, "device or config index out of range");
     std::lock_guard<std::mutex> lk(mu);
-    int &slot = cache[dev][c->precision][index][fine ? 3 : mode][pot ? 1 : 0];
+    int &slot = cache[dev][c->precision][index][tiles ? 2 + tiles : mode][pot ? 1 : 0];
     if (slot == 0) {
         int b = 0;
-        const occupancy_fn occ = fine ? c->occupancy_fine[pot ? 1 : 0] : c->occupancy[mode][pot ? 1 : 0];
+        const occupancy_fn occ = (tiles == kPlain  ? c->occupancy_plain
+                                  : tiles == kFine ? c->occupancy_fine
+                                                   : c->occupancy[mode])[pot ? 1 : 0];
         rc = check_cuda((cudaError_t)occ(&b), "cudaOccupancyMaxActiveBlocksPerMultiprocessor");
         if (rc) return rc;
         if (b < 1) return fail(GRAV_ECUDA, "force kernel cannot be resident on an SM");
@@ -166,20 +172,32 @@ int grid_for(const EvalConfig *c, int index, int mode, bool fine, bool pot, int 
 // twice the configuration's sources to a tile.  Where that leaves fewer work
 // items (target block x tile) than two rounds of the resident CTAs and the
 // sources may be split over them, the items count more than the cost per tile:
-// tiles of the configuration's size (2011 elements 592 -> 470 us; 12289 elements
-// 3.4 ms with the large tiles, 4.2 ms with the small ones).
-constexpr int64_t kFinePairs = 1LL << 25;
+// tiles of the configuration's size (2011 elements 592 -> 470 us; 5000
+// 1.24 ms on small tiles, 5793 2.80 ms on large ones; 12289 elements 3.4 ms with the
+// large tiles, 4.2 ms with the small ones).
+constexpr int64_t kFinePairs = 1LL << 26;
 
-bool fine_tiles(const grav_params *p, const EvalConfig *c, int mode, int64_t n_src, int64_t n_idx_max)
+int tile_kind(const grav_params *p, const EvalConfig *c, int mode, int64_t n_src, int64_t n_idx_max)
 {
-    return c->precision == GRAV_F64 && mode == kModeOpen && p->max_split != 1 &&
-           n_src * n_idx_max < kFinePairs;
+    if (c->precision != GRAV_F64 || mode != kModeOpen || p->max_split == 1) return kNominal;
+    // The smallest keep FP64 pair terms: a sub-block of 32 of a few thousand
+    // elements is so long that most pairs of a concentrated system count as
+    // close and are summed in FP64 anyway.  Up to two items (target block x
+    // tile) an SM, and from three, the two-part kernel's residency, to four, where
+    // its second round is nearly empty (Plummer, FP64 / two-part: 500 elements 234 /
+    // 288 us, 2139 409 / 460, 2500 591 / 485, 2900 753 / 833, 3500 1172 / 895).
+    int sms = 0;
+    if (device_sm_count(&sms) != GRAV_OK) sms = 152;
+    const int64_t BT = (int64_t)c->threads * c->kt;
+    const int64_t items = ((n_idx_max + BT - 1) / BT) * ((n_src + c->s - 1) / c->s);
+    if (items <= 2 * sms || (items > 3 * sms && items <= 4 * sms)) return kPlain;
+    return n_src * n_idx_max < kFinePairs ? kFine : kNominal;
 }
 
 // Sources per packed tile and bytes per source of the packed tiles.
-int64_t tile_sources(const EvalConfig *c, int mode, bool fine)
+int64_t tile_sources(const EvalConfig *c, int mode, int tiles)
 {
-    return c->precision == GRAV_F64 && mode == kModeOpen && !fine ? 2 * c->s : c->s;
+    return c->precision == GRAV_F64 && mode == kModeOpen && tiles == kNominal ? 2 * c->s : c->s;
 }
 
 int64_t source_bytes(const EvalConfig *c, int mode)
@@ -203,14 +221,23 @@ int make_layout(const grav_params *p, const EvalConfig *c, int64_t n_src, int64_
     int sms = 0;
     int rc = device_sm_count(&sms);
     if (rc) return rc;
-    const int64_t S = tile_sources(c, mode, fine_tiles(p, c, mode, n_src, n_idx_max));
+    const int tiles = tile_kind(p, c, mode, n_src, n_idx_max);
+    const int64_t S = tile_sources(c, mode, tiles);
     const int64_t BT = (int64_t)c->threads * c->kt;
     const int NC = p->want_pot ? kNCPot : kNC;
     L->max_split = p->max_split > 0 ? p->max_split : kDefaultMaxSplit;
     L->n_tiles = (n_src + S - 1) / S;
     L->geo_off = 0;
-    L->src_off = round_up(L->n_tiles * (int64_t)sizeof(TileGeom), 256);
-    L->lo_off = L->src_off + round_up(L->n_tiles * S * source_bytes(c, mode), 256);
+    int64_t geo_room = L->n_tiles, src_room = L->n_tiles * S * source_bytes(c, mode);
+    if (c->precision == GRAV_F64 && mode == kModeOpen) {
+        // the same room for every kind of tile, so that a workspace sized for
+        // more targets also does for fewer
+        geo_room = (n_src + c->s - 1) / c->s;
+        src_room = std::max(geo_room * c->s * 64,
+                            round_up(n_src, 2 * (int64_t)c->s) * kDfBytesPerSource);
+    }
+    L->src_off = round_up(geo_room * (int64_t)sizeof(TileGeom), 256);
+    L->lo_off = L->src_off + round_up(src_room, 256);
     const int64_t lo_bytes = (c->precision == GRAV_MIXED) ? L->n_tiles * kLoPlanes * S * 4 : 0;
     L->part_off = L->lo_off + round_up(lo_bytes, 256);
     const int64_t n_tb_max = (n_idx_max + BT - 1) / BT;
@@ -334,13 +361,13 @@ int eval_single(const char *who, const grav_params *p, bool soft, int64_t n_src,
             index = kFewMixed;
         } else if (n_idx_dev) {
             few = f;
-            rc = grid_for(few, kFewMixed, mode, false, want_pot, &few_grid);
+            rc = grid_for(few, kFewMixed, mode, kNominal, want_pot, &few_grid);
             if (rc) return rc;
         }
     }
     int grid = 0;
-    const bool fine = fine_tiles(p, c, mode, n_src, n_idx_max);
-    rc = grid_for(c, index, mode, fine, want_pot, &grid);
+    const int tiles = tile_kind(p, c, mode, n_src, n_idx_max);
+    rc = grid_for(c, index, mode, tiles, want_pot, &grid);
     if (rc) return rc;
 
     char *ws = static_cast<char *>(workspace);
@@ -387,7 +414,7 @@ int eval_single(const char *who, const grav_params *p, bool soft, int64_t n_src,
     }
 
     cudaStream_t st = as_stream(stream);
-    (fine ? c->pack_fine : c->pack[mode])(n_src, pos, vel, mass, const_cast<TileGeom *>(a.geo), const_cast<void *>(a.src), flags_dev,
+    (tiles == kPlain ? c->pack_plain : tiles == kFine ? c->pack_fine : c->pack[mode])(n_src, pos, vel, mass, const_cast<TileGeom *>(a.geo), const_cast<void *>(a.src), flags_dev,
             const_cast<float *>(a.src_lo), (int)L.n_tiles, st);
     rc = check_launch("grav_eval/pack");
     if (rc) return rc;
@@ -411,7 +438,7 @@ int eval_single(const char *who, const grav_params *p, bool soft, int64_t n_src,
         a.few_grid = few_grid;
         a.few_bt = few->threads * few->kt;
     }
-    (fine ? c->launch_fine : c->launch[mode])[want_pot ? 1 : 0](a, grid, st);
+    (tiles == kPlain ? c->launch_plain : tiles == kFine ? c->launch_fine : c->launch[mode])[want_pot ? 1 : 0](a, grid, st);
     rc = check_launch("grav_eval/eval");
     if (rc) return rc;
     const int32_t BT = c->threads * c->kt;
@@ -591,7 +618,7 @@ struct BatchLayout {
 BatchLayout batch_layout(const EvalConfig *c, int mode, int32_t n_sys, int64_t n_total)
 {
     BatchLayout L;
-    const int64_t S = tile_sources(c, mode, false);
+    const int64_t S = tile_sources(c, mode, kNominal);
     L.max_tiles = (n_total + S - 1) / S + n_sys;
     int64_t o = 0;
     L.hdr = o;
@@ -759,7 +786,7 @@ extern "C" int grav_eval_batched(const grav_params *p, int32_t n_sys, const grav
     cudaStream_t st = as_stream(stream);
     const int32_t BT = c->threads * c->kt;
     rc = launch_batch_plan(b, idx, n_idx_dev, n_idx_max, n_total,
-                           (int32_t)tile_sources(c, mode, false), BT, p->box, flags_dev, st);
+                           (int32_t)tile_sources(c, mode, kNominal), BT, p->box, flags_dev, st);
     if (rc) return rc;
     c->pack_batched[p->box > 0.0 ? 1 : 0](b, pos, vel, mass, const_cast<TileGeom *>(a.geo), const_cast<void *>(a.src),
                     flags_dev, const_cast<float *>(a.src_lo), (int)L.max_tiles, st);
