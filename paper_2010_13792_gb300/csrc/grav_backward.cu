@@ -249,7 +249,7 @@ __device__ __forceinline__ bool bwd_df_item(const BwdArgs &a, BwdDfSmem<NT, S> &
     int cnt = 0;
     for (int t = t_begin; t < t_end; ++t) {
         const int s = (t - t_begin) % NSTAGE;
-        const bool got = mbar_wait_bounded(&sm.bar[s], (ring.parity >> s) & 1u, a.flags);
+        const bool got = mbar_wait_warp(&sm.bar[s], (ring.parity >> s) & 1u, a.flags);
         if (got)
             ring.parity ^= 1u << s;
         else
@@ -333,7 +333,7 @@ __device__ __forceinline__ bool bwd_df_item(const BwdArgs &a, BwdDfSmem<NT, S> &
             }
         }
         __syncwarp();
-        if (*(volatile int *)&sm.abort_flag) break;
+        if (__any_sync(0xffffffffu, *(volatile int *)&sm.abort_flag)) break;
     }
     __syncthreads();   // every warp is out of the tile loop: a uniform status
     if (cnt > 0) bwd_df_flush(a.pos, a.a_bar, h, i, list, cnt, sum, NT);

@@ -180,6 +180,15 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t *bar, uint32_t parity
     return false;
 }
 
+// The same for a warp whose lanes branch on the status or vote afterwards: true
+// only if no lane gave up.  The lanes poll on their own, so a copy that lands
+// while some have run out of polls leaves them with different answers; a vote
+// of the full warp inside such a branch would wait for lanes that never come.
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t *bar, uint32_t parity, int32_t *flags)
+{
+    return __all_sync(0xffffffffu, mbar_wait_bounded(bar, parity, flags));
+}
+
 // Tidal timestep, Eq. (tidaltimestep): sqrt(eta) * (||T||_F^2 / 6)^(-1/4),
 // ||T||^2 summed in the fixed order xx, yy, zz, then 2xy^2, 2xz^2, 2yz^2,
 // every operation correctly rounded (no contraction); +inf for T = 0.

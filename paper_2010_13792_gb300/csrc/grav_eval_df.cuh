@@ -245,7 +245,7 @@ __device__ __forceinline__ bool df_item(const EvalArgs &a, DfSmem<NT, S, POT> &s
 
     for (int t = t_begin; t < t_end; ++t) {
         const int s = (t - t_begin) % NSTAGE;
-        const bool got = mbar_wait_bounded(&sm.bar[s], (ring.parity >> s) & 1u, a.flags);
+        const bool got = mbar_wait_warp(&sm.bar[s], (ring.parity >> s) & 1u, a.flags);
         if (got)
             ring.parity ^= 1u << s;
         else
@@ -342,7 +342,7 @@ __device__ __forceinline__ bool df_item(const EvalArgs &a, DfSmem<NT, S, POT> &s
             }
         }
         __syncwarp();
-        if (*(volatile int *)&sm.abort_flag) break;
+        if (__any_sync(0xffffffffu, *(volatile int *)&sm.abort_flag)) break;
     }
     // warps leave the tile loop at different times: a uniform status
     __syncthreads();
