@@ -372,9 +372,14 @@ constexpr float kDfRange = 32768.0f;   // targets beyond this many L from a tile
 // its sources) are listed for FP64, and so are softened pairs.
 constexpr float kDfNear = 0.42f;
 constexpr int kDfList = 64;            // room for two sub-blocks per target
+// Least r^2 / L^2 in two parts: from there m r^-5 stays below 2^110 in FP32.  L is
+// at least 2^-10 of the tile's distance from the origin, so a tile a billion
+// times smaller than that distance has pairs below it (r^-5 ran over in the
+// jerk and the tidal tensor); it is right for targets farther away.
+constexpr float kDfLeast2 = 0x1p-44f;
 
 struct DfClass {
-    uint32_t direct;   // sub-blocks summed in FP64 (softening wider than half their diagonal)
+    uint32_t direct;   // sub-blocks summed in FP64 (softening wider than half their diagonal, kDfLeast2)
     uint32_t close;    // sub-blocks with listed pairs
     float rmin2;       // least r^2 of the pairs left to this lane's target
     float floor2;      // least listing radius (squared)
@@ -425,6 +430,11 @@ __device__ __forceinline__ DfClass df_classify(const float *tile, const DfHead &
         }
         gap2 *= 1.0f - 0x1p-18f;
         const float diag2 = df_diagonal2(box), thr2 = df_radius2(k, diag2);
+        const float least2 = fmaxf(gap2, thr2 * (1.0f - 0x1p-10f));
+        if (__any_sync(0xffffffffu, live && least2 < kDfLeast2)) {
+            k.direct |= 1u << q;
+            continue;
+        }
         if (__any_sync(0xffffffffu, live && !(gap2 > thr2))) {
             // (mostly softened pairs: no list)
             if (hl * hl > 0.25f * diag2) {
@@ -434,7 +444,7 @@ __device__ __forceinline__ DfClass df_classify(const float *tile, const DfHead &
             k.close |= 1u << q;
         }
         // (lanes without a target: any window)
-        if (live) k.rmin2 = fminf(k.rmin2, fmaxf(gap2, thr2 * (1.0f - 0x1p-10f)));
+        if (live) k.rmin2 = fminf(k.rmin2, least2);
     }
     return k;
 }
