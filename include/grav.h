@@ -63,9 +63,14 @@ extern "C" {
 #define GRAV_FLAG_OVERFLOW  16 /* a tree build or walk exceeded its node bound (not expected) */
 
 /* Arithmetic of the force sums. */
-#define GRAV_F64   0  /* FP64 results: pair terms in FP64, or (open boundaries) in two-part
-                         FP32 with the closest pairs and the final sums in FP64, with the
-                         error of the FP64 sums (csrc/grav_df.cuh) */
+#define GRAV_F64   0  /* FP64 inputs, sums and results.  Pair terms in FP64, or (open
+                         boundaries) in two-part FP32, good to some 8e-15 of themselves,
+                         where many like terms of a source tile average that to 1e-15 of
+                         the tile's sum; the closest pairs, sources that carry their tile,
+                         terms that cancel and systems of up to 128 elements stay in FP64
+                         (csrc/grav_df.cuh).  An output is within about 2e-15 of the sum of
+                         its terms' magnitudes (the jerk's taken with the largest relative
+                         velocity), as with FP64 pair terms throughout. */
 #define GRAV_MIXED 1  /* FP64 positions offset to FP32 per source tile, FP32 pair
                          arithmetic, compensated FP32 tile sums, FP64 final sums */
 

@@ -284,9 +284,11 @@ __device__ __forceinline__ bool bwd_df_item(const BwdArgs &a, BwdDfSmem<NT, S> &
                             __syncwarp();
                         }
                         const int64_t j0 = g.first + kDfSub * q;
-                        const int real = min(kDfSub, head.count - kDfSub * q);
+                        // (not padding, not the heavy ones)
+                        const uint32_t light = (0xffffffffu >> (kDfSub - min(kDfSub, head.count - kDfSub * q))) &
+                                               ~df_heavy<S>(tile, q);
                         auto add = [&](int j) {
-                            if (live && j < real && j0 + j != i) list[cnt++] = (int32_t)(j0 + j);
+                            if (live && (light >> j & 1u) && j0 + j != i) list[cnt++] = (int32_t)(j0 + j);
                         };
                         bwd_df_loop<true>(Pq, tg, w3, w2,
                                           df_radius2(k, df_diagonal2(tile + kDfHeader + 6 * q)), sums, add);
@@ -300,19 +302,17 @@ __device__ __forceinline__ bool bwd_df_item(const BwdArgs &a, BwdDfSmem<NT, S> &
                 for (int c = 0; c < kNB; ++c)
                     acc[c] = df_value(sums[c], c == MBS ? w2 : w3, n1, n2, c == MBS ? u2 : u3);
             }
-            if (k.direct) {
+            for (int q = 0; q < n_sub; ++q) {
+                uint32_t marks = df_fp64_sources<S>(tile, k, q, min(kDfSub, head.count - kDfSub * q));
+                if (!marks) continue;
                 const double h2 = h * h, hinv = 1.0 / h;
                 const double hinv3 = hinv * hinv * hinv, hinv5 = hinv3 * hinv * hinv;
-                for (int q = 0; q < n_sub; ++q) {
-                    if (!((k.direct >> q) & 1u)) continue;
-                    const int real = min(kDfSub, head.count - kDfSub * q);
-                    for (int m = 0; m < real; ++m) {
-                        const int64_t j = g.first + kDfSub * q + m;
-                        const double d[3] = {a.pos[3 * j] - xk[0], a.pos[3 * j + 1] - xk[1],
-                                             a.pos[3 * j + 2] - xk[2]};
-                        const double ab[3] = {a.a_bar[3 * j], a.a_bar[3 * j + 1], a.a_bar[3 * j + 2]};
-                        bwd_pair_fp64(d, ab, h2, hinv, hinv3, hinv5, j == i, acc);
-                    }
+                for (; marks; marks &= marks - 1u) {
+                    const int64_t j = g.first + kDfSub * q + __ffs(marks) - 1;
+                    const double d[3] = {a.pos[3 * j] - xk[0], a.pos[3 * j + 1] - xk[1],
+                                         a.pos[3 * j + 2] - xk[2]};
+                    const double ab[3] = {a.a_bar[3 * j], a.a_bar[3 * j + 1], a.a_bar[3 * j + 2]};
+                    bwd_pair_fp64(d, ab, h2, hinv, hinv3, hinv5, j == i, acc);
                 }
             }
             bwd_add_sums(sum, NT, acc);

@@ -24,10 +24,11 @@
 //     a second time at the unit of a smaller constant, and what then remains
 //     joins the product's low part in an FP32 sum.  Nothing but that last sum
 //     is rounded, and it is 2^20 and more below the total even where the window
-//     is a thousand times wider than the sum (unequal masses).
-// A pair comes out good to about 8e-15 (rms, its force), and thousands of them
-// average; the pairs closest to a target, whose rounding would not, are listed
-// and summed in FP64.
+//     is a thousand times wider than the sum.
+// A pair comes out good to about 8e-15 (rms, its force; FP64 3e-16), and the
+// terms of a tile average that.  What would not average is summed in FP64: the
+// pairs closest to a target (listed), sources that carry a tile and tiles whose
+// terms cancel (kDfAverage).
 #pragma once
 
 #include "grav_common.cuh"
@@ -35,13 +36,16 @@
 namespace grav {
 
 // Words of a packed tile of S sources: an 8-word header, the boxes of its
-// sub-blocks of 32 sources (lo, hi in units of L, rounded outward), S/2
+// sub-blocks of 32 sources (lo, hi in units of L, rounded outward), a word per
+// sub-block that marks its heavy sources (a multiple of 4 words so far), S/2
 // records of 28 floats (two sources side by side: xh yh zh xl yl zl, the same
-// of the velocity, mh ml).
+// of the velocity, mh ml; heavy sources and padding with mass and velocity 0).
 constexpr int kDfSub = 32;
 constexpr int kDfHeader = 8;
 template <int S>
-constexpr int df_records() { return kDfHeader + 6 * (S / kDfSub); }
+constexpr int df_heavies() { return kDfHeader + 6 * (S / kDfSub); }
+template <int S>
+constexpr int df_records() { return (df_heavies<S>() + S / kDfSub + 3) / 4 * 4; }
 template <int S>
 constexpr int df_words() { return df_records<S>() + 14 * S; }
 template <int S>
@@ -54,10 +58,10 @@ static_assert(df_bytes<64>() <= df_stride<64>() && df_bytes<128>() <= df_stride<
               df_bytes<256>() <= df_stride<256>() && df_stride<64>() % 16 == 0, "DF tile stride");
 
 struct DfHead {
-    double munit;      // M: the largest |m| (1 if all are 0)
+    double munit;      // M: the largest |m| but for the heavy ones (1 if all are 0)
     float ext[3];      // half extents / L, rounded up
     int16_t el, ev;    // units: L = 2^el >= half extent, V = 2^ev > |v'|
-    int16_t ok;        // 0: out of the ranges above, the tile is summed in FP64
+    int16_t ok;        // 0: the tile is summed in FP64 (out of range, or its terms do not average)
     int16_t count;     // sources in the tile
     int32_t pad;
 };
@@ -76,41 +80,80 @@ __device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y
 // a - b, rounded once
 __device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, dup2(-1.0f), a); }
 
+// Sources that carry a tile.  A two-part pair term is good to some 8e-15 of
+// itself, thirty times FP64's rounding; the sums are as good as FP64's where many
+// like terms average it away, and not where a few terms carry a sum, nor where the
+// windows, which the largest attribute sets, belong to a source that the target
+// does not sum (itself): terms below 2^-42 of the window are plain FP32.  So
+// with w the masses (and the |v'|, or the a_bar) of the tile:
+//   * the tile averages if sum w^2 <= (sum w)^2 / K, the largest w left out of
+//     the right side (a target does not sum itself), K = 64: a spread of
+//     masses, up to 64 equal ones (fewer in a ragged last tile);
+//   * otherwise the sources above sum w / (2 K + 2) are heavy, at most 2 K + 3 of
+//     them: they are summed in FP64, and the rest averages, since its sum of
+//     squares is at most its largest times its sum, sum w^2 <= 2 (sum w)^2 / (2 K + 2);
+//   * a tile whose w cancel (|sum w| < sum |w| / 2, an a_bar of random signs) is
+//     summed in FP64 altogether, and so are systems of up to 128 elements.
+// Measured (rms error of the acceleration; FP64 pairs / two parts alone / with
+// this rule): 10000-element Plummer sphere, masses from 0.1 to 100 with their
+// number falling as m^-2.35 1.7e-16 / 9.9e-16 / 2.4e-16, over 14 decades 2.2e-16 /
+// 1.1e-15 / 1.4e-16; one mass of 1 among 299 of 1e-12, at it, 3.8e-16 / 3.1e-9 /
+// 6.8e-16; the adjoint's largest error for a random a_bar 3e-15 / 6e-14 / 3e-15.
+// 16384 elements: 4.4 ms, with that mass function 5.1 ms.
+constexpr int kDfAverage = 64;
+constexpr int kDfFewest = 128;
+
+// (the larger side of the rule: heavier than this)
+__device__ __forceinline__ float df_heavy_line(float net, float gross, float squares, float K, bool &ok)
+{
+    if (squares * K <= net * net) return __int_as_float(0x7f800000);
+    if (gross > 2.0f * net) ok = false;
+    return net / (2.0f * K + 2.0f);
+}
+
 // Packs one tile (one CTA of S threads, thread j its source): `x` the FP64
 // offset from the tile centre, `v` the velocity relative to the tile's
-// velocity centre (or the adjoint's a_bar), m the mass; `half` the tile's half
-// extents.  Padding sources (!ok) copy the place of their sub-block's first
-// source with zero mass.  A warp is a sub-block.
-template <int S>
-__device__ __forceinline__ void df_pack(void *tile, int j, bool ok, int count, const double x[3],
+// velocity centre (ADJ: the adjoint's a_bar), m the mass; `half` the tile's half
+// extents; `alone`: the system has no other tile.  Padding sources (!ok) copy the
+// place of their sub-block's first source with zero mass.  A warp is a sub-block.
+template <int S, bool ADJ>
+__device__ __forceinline__ void df_pack(void *tile, int j, bool ok, int count, bool alone, const double x[3],
                                         const double v[3], double m, const double half[3], double cmax)
 {
-    __shared__ uint32_t wmax[3][S / 32];
+    constexpr int W = S / 32;
+    __shared__ uint32_t wtop[2][W], wlight[3][W];
+    __shared__ int wat[2][W];
+    __shared__ float wsum[8][W];
     const int lane = j & 31, wid = j >> 5;
-    uint32_t hv = 0, hm = 0, lm = 0;
+    // the largest mass and velocity (by the high words), and who has them
+    uint32_t hv = 0, hm = 0;
     if (ok) {
 #pragma unroll
         for (int c = 0; c < 3; ++c) hv = max(hv, (uint32_t)__double2hiint(v[c]) & 0x7fffffffu);
         hm = (uint32_t)__double2hiint(m) & 0x7fffffffu;
-        lm = (uint32_t)__double2loint(m);
     }
-    hv = __reduce_max_sync(0xffffffffu, hv);
-    const uint32_t top = __reduce_max_sync(0xffffffffu, hm);
-    lm = __reduce_max_sync(0xffffffffu, hm == top ? lm : 0u);
-    hm = top;
-    if (lane == 0) {
-        wmax[0][wid] = hv;
-        wmax[1][wid] = hm;
-        wmax[2][wid] = lm;
+    {
+        const uint32_t tm = __reduce_max_sync(0xffffffffu, hm), tv = __reduce_max_sync(0xffffffffu, hv);
+        const int am = __ffs(__ballot_sync(0xffffffffu, ok && hm == tm)) - 1;
+        const int av = __ffs(__ballot_sync(0xffffffffu, ok && hv == tv)) - 1;
+        if (lane == 0) {
+            wtop[0][wid] = tm;
+            wtop[1][wid] = tv;
+            wat[0][wid] = am;
+            wat[1][wid] = av;
+        }
     }
     __syncthreads();
+    uint32_t top[2] = {0u, 0u};
+    int at[2] = {-1, -1};
 #pragma unroll
-    for (int w = 0; w < S / 32; ++w) {
-        hv = max(hv, wmax[0][w]);
-        const uint32_t h2 = wmax[1][w], l2 = wmax[2][w];
-        lm = h2 > hm ? l2 : h2 == hm ? max(lm, l2) : lm;
-        hm = max(hm, h2);
-    }
+    for (int w = 0; w < W; ++w)
+#pragma unroll
+        for (int c = 0; c < 2; ++c)
+            if (wat[c][w] >= 0 && (at[c] < 0 || wtop[c][w] > top[c])) {
+                top[c] = wtop[c][w];
+                at[c] = 32 * w + wat[c][w];
+            }
     uint32_t hx = 0;
 #pragma unroll
     for (int c = 0; c < 3; ++c) hx = max(hx, (uint32_t)__double2hiint(half[c]) & 0x7fffffffu);
@@ -120,14 +163,72 @@ __device__ __forceinline__ void df_pack(void *tile, int j, bool ok, int count, c
     DfHead h;
     int el = max(exponent_above(hx), exponent_above(hc) - 10);
     if (hx == 0 && hc == 0) el = 0;
-    const int ev = hv == 0 ? 0 : exponent_above(hv);
-    const int em = hm == 0 ? 0 : exponent_above(hm);
-    h.ok = hx < 0x7ff00000u && hv < 0x7ff00000u && hm < 0x7ff00000u && abs(el) <= 150 &&
-           abs(ev) <= 150 && abs(em) <= 150;
+    const int em = top[0] == 0 ? 0 : exponent_above(top[0]), ev = top[1] == 0 ? 0 : exponent_above(top[1]);
+    bool good = hx < 0x7ff00000u && top[0] < 0x7ff00000u && top[1] < 0x7ff00000u && abs(el) <= 150 &&
+                abs(em) <= 150 && abs(ev) <= 150 && !(alone && count <= kDfFewest);
     el = max(-150, min(150, el));
     h.el = (int16_t)el;
-    h.ev = (int16_t)max(-150, min(150, ev));
-    h.munit = h.ok && hm != 0 ? __hiloint2double((int)hm, (int)lm) : 1.0;
+    // heavy sources
+    float w = 0.0f, u[3] = {0.0f, 0.0f, 0.0f};
+    if (ok && good) {
+        const double im = pow2d(-em), iv = pow2d(-ev);
+        w = __double2float_rn(__dmul_rn(m, im));
+#pragma unroll
+        for (int c = 0; c < 3; ++c) u[c] = __double2float_rn(__dmul_rn(v[c], iv));
+    }
+    const float uu = fmaf(u[0], u[0], fmaf(u[1], u[1], u[2] * u[2])), un = sqrtf(uu);
+    const bool not_m = j != at[0], not_v = j != at[1];
+    float sum[8] = {not_m ? w : 0.0f,    not_m ? fabsf(w) : 0.0f, w * w,
+                    not_v ? u[0] : 0.0f, not_v ? u[1] : 0.0f,     not_v ? u[2] : 0.0f,
+                    not_v ? un : 0.0f,   uu};
+    constexpr int kFirst = ADJ ? 3 : 0;
+#pragma unroll
+    for (int q = kFirst; q < 8; ++q) {
+        if (!ADJ && q >= 3 && q < 6) continue;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) sum[q] += __shfl_xor_sync(0xffffffffu, sum[q], o);
+        if (lane == 0) wsum[q][wid] = sum[q];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int q = kFirst; q < 8; ++q) {
+        if (!ADJ && q >= 3 && q < 6) continue;
+        sum[q] = 0.0f;
+#pragma unroll
+        for (int k = 0; k < W; ++k) sum[q] += wsum[q][k];
+    }
+    const float K = fminf((float)kDfAverage, 0.5f * (float)count);
+    const float net_v = ADJ ? sqrtf(fmaf(sum[3], sum[3], fmaf(sum[4], sum[4], sum[5] * sum[5]))) : sum[6];
+    bool heavy = un > df_heavy_line(net_v, sum[6], sum[7], K, good);
+    if (!ADJ) heavy = fabsf(w) > df_heavy_line(fabsf(sum[0]), sum[1], sum[2], K, good) || heavy;
+    // the units are those of the others
+    const uint32_t marks = __ballot_sync(0xffffffffu, heavy);
+    {
+        uint32_t lm = (uint32_t)__double2loint(m);
+        if (!ok || heavy) hv = hm = lm = 0;
+        const uint32_t tv = __reduce_max_sync(0xffffffffu, hv), tm = __reduce_max_sync(0xffffffffu, hm);
+        lm = __reduce_max_sync(0xffffffffu, hm == tm ? lm : 0u);
+        if (lane == 0) {
+            wlight[0][wid] = tv;
+            wlight[1][wid] = tm;
+            wlight[2][wid] = lm;
+        }
+    }
+    __syncthreads();
+    hv = hm = 0;
+    uint32_t lm = 0;
+#pragma unroll
+    for (int k = 0; k < W; ++k) {
+        hv = max(hv, wlight[0][k]);
+        const uint32_t h2 = wlight[1][k], l2 = wlight[2][k];
+        lm = h2 > hm ? l2 : h2 == hm ? max(lm, l2) : lm;
+        hm = max(hm, h2);
+    }
+    // (the sums above are FP32: they say nothing of what lies 2^96 below)
+    good = good && (hm == 0 || exponent_above(hm) >= em - 96) && (hv == 0 || exponent_above(hv) >= ev - 96);
+    h.ok = good;
+    h.ev = (int16_t)(good && hv != 0 ? exponent_above(hv) : 0);
+    h.munit = good && hm != 0 ? __hiloint2double((int)hm, (int)lm) : 1.0;
     h.count = (int16_t)count;
     h.pad = 0;
     const double il = pow2d(-el);
@@ -138,6 +239,7 @@ __device__ __forceinline__ void df_pack(void *tile, int j, bool ok, int count, c
     const double iv = pow2d(-h.ev);
     float *rec = out + df_records<S>() + 28 * (j >> 1) + (j & 1);
     float *box = out + kDfHeader + 6 * wid;
+    if (lane == 0) reinterpret_cast<uint32_t *>(out)[df_heavies<S>() + wid] = good ? marks : 0u;
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
         const double s = __shfl_sync(0xffffffffu, __dmul_rn(x[c], il), ok ? lane : 0);
@@ -154,15 +256,15 @@ __device__ __forceinline__ void df_pack(void *tile, int j, bool ok, int count, c
             box[c] = lo;
             box[3 + c] = hi;
         }
-        const double u = ok ? __dmul_rn(v[c], iv) : 0.0;
-        const float vh = __double2float_rn(u);
+        const double vu = ok && !heavy ? __dmul_rn(v[c], iv) : 0.0;
+        const float vh = __double2float_rn(vu);
         rec[12 + 2 * c] = vh;
-        rec[18 + 2 * c] = __double2float_rn(__dsub_rn(u, (double)vh));
+        rec[18 + 2 * c] = __double2float_rn(__dsub_rn(vu, (double)vh));
     }
-    const double w = ok ? __ddiv_rn(m, h.munit) : 0.0;
-    const float mh = __double2float_rn(w);
+    const double mw = ok && !heavy ? __ddiv_rn(m, h.munit) : 0.0;
+    const float mh = __double2float_rn(mw);
     rec[24] = mh;
-    rec[26] = __double2float_rn(__dsub_rn(w, (double)mh));
+    rec[26] = __double2float_rn(__dsub_rn(mw, (double)mh));
 }
 
 // A target against one tile: offset from the tile centre in units of L, in
@@ -384,6 +486,20 @@ struct DfClass {
     float rmin2;       // least r^2 of the pairs left to this lane's target
     float floor2;      // least listing radius (squared)
 };
+
+// The heavy sources of sub-block q.
+template <int S>
+__device__ __forceinline__ uint32_t df_heavy(const float *tile, int q)
+{
+    return reinterpret_cast<const uint32_t *>(tile)[df_heavies<S>() + q];
+}
+
+// The sources of a sub-block of `real` that go to FP64 one by one.
+template <int S>
+__device__ __forceinline__ uint32_t df_fp64_sources(const float *tile, const DfClass &k, int q, int real)
+{
+    return (k.direct >> q) & 1u ? 0xffffffffu >> (kDfSub - real) : df_heavy<S>(tile, q);
+}
 
 __device__ __forceinline__ float df_diagonal2(const float *box)
 {

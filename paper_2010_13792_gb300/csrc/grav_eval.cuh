@@ -376,7 +376,8 @@ __device__ __forceinline__ void pack_tile(int t, int64_t first, int64_t end,
                                           const double *__restrict__ vel,
                                           const double *__restrict__ mass,
                                           TileGeom *__restrict__ geo, void *__restrict__ src,
-                                          int32_t *flags, float *__restrict__ src_lo = nullptr)
+                                          int32_t *flags, float *__restrict__ src_lo = nullptr,
+                                          bool alone = false)
 {
     constexpr int NV = VOFF ? 6 : 3;      // boxes of the positions and, with VOFF, the velocities
     __shared__ double mm[2 * NV];
@@ -473,8 +474,8 @@ __device__ __forceinline__ void pack_tile(int t, int64_t first, int64_t end,
         for (int c = 0; c < 3; ++c)
             half[c] = fmax(__dsub_ru(mm[2 * c + 1], cc[c]), __dsub_ru(cc[c], mm[2 * c]));
         const double cmax = fmax(fabs(cc[0]), fmax(fabs(cc[1]), fabs(cc[2])));
-        df_pack<S>(static_cast<char *>(src) + (int64_t)t * df_stride<S>(), j, ok, (int)(end - first < S ? end - first : S),
-                   off, vo, m, half, cmax);
+        df_pack<S, !VOFF>(static_cast<char *>(src) + (int64_t)t * df_stride<S>(), j, ok,
+                          (int)(end - first < S ? end - first : S), alone, off, vo, m, half, cmax);
     } else {
         D4 *tile = static_cast<D4 *>(src) + (int64_t)t * 2 * S;
         D4 pm, pv;
@@ -512,7 +513,7 @@ pack_tiles_kernel(int64_t n_src, const double *__restrict__ pos, const double *_
     const int64_t first = (int64_t)blockIdx.x * S;
     const int64_t end = first + S < n_src ? first + S : n_src;
     pack_tile<S, MIXED, VOFF, PAIR, DF>(blockIdx.x, first, end, pos, vel, mass, geo, src, flags,
-                                        src_lo);
+                                        src_lo, n_src <= S);
 }
 
 // ---------------------------------------------------------------------------
@@ -1925,7 +1926,8 @@ pack_tiles_batched_kernel(const BatchView b, const double *__restrict__ pos,
     const int64_t first = b.sys[lo].offset + (int64_t)(t - b.tile_off[lo]) * S;
     const int64_t sys_end = b.sys[lo].offset + b.sys[lo].n;
     const int64_t end = first + S < sys_end ? first + S : sys_end;
-    pack_tile<S, MIXED, VOFF, PAIR, DF>(t, first, end, pos, vel, mass, geo, src, flags, src_lo);
+    pack_tile<S, MIXED, VOFF, PAIR, DF>(t, first, end, pos, vel, mass, geo, src, flags, src_lo,
+                                        b.sys[lo].n <= S);
 }
 
 // ---------------------------------------------------------------------------

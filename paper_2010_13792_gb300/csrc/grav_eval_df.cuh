@@ -180,20 +180,21 @@ __device__ __noinline__ void df_flush(const double *__restrict__ pos, const doub
     }
 }
 
-// count sources from element `first` in FP64 from the caller's arrays (every
-// lane reads the same source): sub-blocks inside the softening, tiles out of
-// the two-part ranges.
+// The marked sources of the sub-block at element `first` in FP64 from the
+// caller's arrays (every lane reads the same source): heavy sources, sub-blocks
+// inside the softening, tiles out of the two-part ranges.
 template <bool POT>
-__device__ __forceinline__ void df_fp64_loop(const EvalArgs &a, const TileGeom &g, int64_t first, int count,
-                                             const double xi[3], int64_t ti, double acc[kNCPot])
+__device__ __forceinline__ void df_fp64_loop(const EvalArgs &a, const TileGeom &g, int64_t first,
+                                             uint32_t marks, const double xi[3], int64_t ti,
+                                             double acc[kNCPot])
 {
     const double h2 = a.h * a.h, hinv = 1.0 / a.h;
     const double hinv3 = hinv * hinv * hinv;
     const double hinv5 = hinv3 * hinv * hinv;
     const double cv[3] = {(double)g.cv[0], (double)g.cv[1], (double)g.cv[2]};
 #pragma unroll 2
-    for (int k = 0; k < count; ++k) {
-        const int64_t j = first + k;
+    for (; marks; marks &= marks - 1u) {
+        const int64_t j = first + __ffs(marks) - 1;
         const double dx = a.pos[3 * j] - xi[0], dy = a.pos[3 * j + 1] - xi[1], dz = a.pos[3 * j + 2] - xi[2];
         double mf, mg, mp;
         df_pair_terms<POT, false>(fma(dx, dx, fma(dy, dy, dz * dz)), a.mass[j], h2, hinv, hinv3, hinv5, mf, mg,
@@ -313,10 +314,10 @@ __device__ __forceinline__ bool df_item(const EvalArgs &a, DfSmem<NT, S, POT> &s
                 // beyond the softening m f = m g' r^2
                 acc[FSUM] = __dadd_rn(__dadd_rn(acc[TXX], acc[TYY]), acc[TZZ]);
             }
-            for (int q = 0; q < n_sub; ++q)
-                if ((k.direct >> q) & 1u)
-                    df_fp64_loop<POT>(a, g, g.first + (int64_t)kDfSub * q,
-                                      min(kDfSub, head.count - kDfSub * q), xi, i, acc);
+            for (int q = 0; q < n_sub; ++q) {
+                const uint32_t marks = df_fp64_sources<S>(tile, k, q, min(kDfSub, head.count - kDfSub * q));
+                if (marks) df_fp64_loop<POT>(a, g, g.first + (int64_t)kDfSub * q, marks, xi, i, acc);
+            }
             target_velocity_d(acc, vr);
 #pragma unroll
             for (int c = 0; c < NC; ++c) {
