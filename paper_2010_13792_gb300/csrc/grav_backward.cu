@@ -165,7 +165,7 @@ __device__ __forceinline__ void bwd_pair_fp64(const double d[3], const double ab
     const double ri2 = ri * ri;
     double f = ri * ri2;
     double gp = f * ri2;
-    if (r2 < h2) {
+    if (__double_as_longlong(r2) < __double_as_longlong(h2)) {   // (as df_pair_terms)
         double F, Gp, P;
         spline_kernel<double>(sqrt(r2) * hinv, F, Gp, P);
         f = F * hinv3;
@@ -216,6 +216,46 @@ __device__ __noinline__ void bwd_df_flush(const double *__restrict__ pos, const 
     bwd_add_sums(sum, stride, acc);
 }
 
+// A tile's sources that go to FP64 (reasons: df_fp64_loop of the forward).  Not
+// inlined: its registers are not the two-part loop's (12289 elements of like a_bar
+// 1.74 ms inlined, 1.69 ms; all in FP64 7.24 ms, 7.19 ms; FP64 tiles throughout 7.47 ms).
+template <int S>
+__device__ __noinline__ void bwd_fp64_tile(const double *__restrict__ pos, const double *__restrict__ a_bar,
+                                           double h, const float *tile, uint32_t direct, int64_t first_of_tile,
+                                           int count, double xk, double yk, double zk, int64_t ti,
+                                           double sums[kNB])
+{
+    const DfSoftening hk(h);
+    const double at[3] = {xk, yk, zk};
+    double acc[kNB];
+#pragma unroll
+    for (int c = 0; c < kNB; ++c) acc[c] = sums[c];
+    for (int q = 0; q < (count + kDfSub - 1) / kDfSub; ++q) {
+        const uint32_t marks = df_fp64_sources<S>(tile, direct, q, min(kDfSub, count - kDfSub * q));
+        if (!marks) continue;
+        const int64_t first = first_of_tile + kDfSub * q;
+        const DfMarked s(marks, ti - first);
+        double x[3], b[3];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            x[c] = pos[3 * (first + s.own) + c];
+            b[c] = a_bar[3 * (first + s.own) + c];
+        }
+#pragma unroll 2
+        for (int p = 0; p < s.count; ++p) {
+            double d[3], ab[3];
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                d[c] = __shfl_sync(0xffffffffu, x[c], p) - at[c];
+                ab[c] = __shfl_sync(0xffffffffu, b[c], p);
+            }
+            bwd_pair_fp64(d, ab, hk.h2, hk.hinv, hk.hinv3, hk.hinv5, p == s.self, acc);
+        }
+    }
+#pragma unroll
+    for (int c = 0; c < kNB; ++c) sums[c] = acc[c];
+}
+
 // One item of the FP64 adjoint (structure and reasons: df_item of the forward,
 // grav_eval_df.cuh); false once a bounded wait gave up.
 template <int NT, int S>
@@ -259,9 +299,14 @@ __device__ __forceinline__ bool bwd_df_item(const BwdArgs &a, BwdDfSmem<NT, S> &
             const float *tile = sm.stage[s];
             const DfHead head = *reinterpret_cast<const DfHead *>(tile);
             DfTarget tg;
-            const double il = df_offset(head, g.c, xk, tg);
-            const DfClass k = df_classify(tile, head, tg, live, h, il);
+            DfClass k;
             const int el = head.el, n_sub = (head.count + kDfSub - 1) / kDfSub;
+            if (head.ok) {
+                const double il = df_offset(head, g.c, xk, tg);
+                k = df_classify(tile, head, tg, live, h, il);
+            } else {
+                k.direct = (1u << n_sub) - 1u;
+            }
             double acc[kNB];
 #pragma unroll
             for (int c = 0; c < kNB; ++c) acc[c] = 0.0;
@@ -302,19 +347,9 @@ __device__ __forceinline__ bool bwd_df_item(const BwdArgs &a, BwdDfSmem<NT, S> &
                 for (int c = 0; c < kNB; ++c)
                     acc[c] = df_value(sums[c], c == MBS ? w2 : w3, n1, n2, c == MBS ? u2 : u3);
             }
-            for (int q = 0; q < n_sub; ++q) {
-                uint32_t marks = df_fp64_sources<S>(tile, k, q, min(kDfSub, head.count - kDfSub * q));
-                if (!marks) continue;
-                const double h2 = h * h, hinv = 1.0 / h;
-                const double hinv3 = hinv * hinv * hinv, hinv5 = hinv3 * hinv * hinv;
-                for (; marks; marks &= marks - 1u) {
-                    const int64_t j = g.first + kDfSub * q + __ffs(marks) - 1;
-                    const double d[3] = {a.pos[3 * j] - xk[0], a.pos[3 * j + 1] - xk[1],
-                                         a.pos[3 * j + 2] - xk[2]};
-                    const double ab[3] = {a.a_bar[3 * j], a.a_bar[3 * j + 1], a.a_bar[3 * j + 2]};
-                    bwd_pair_fp64(d, ab, h2, hinv, hinv3, hinv5, j == i, acc);
-                }
-            }
+            if (df_any_fp64<S>(tile, k.direct, n_sub))
+                bwd_fp64_tile<S>(a.pos, a.a_bar, h, tile, k.direct, g.first, head.count, xk[0], xk[1], xk[2], i,
+                                 acc);
             bwd_add_sums(sum, NT, acc);
         }
         // this warp is done reading stage s; the last warp refills it

@@ -496,10 +496,46 @@ __device__ __forceinline__ uint32_t df_heavy(const float *tile, int q)
 
 // The sources of a sub-block of `real` that go to FP64 one by one.
 template <int S>
-__device__ __forceinline__ uint32_t df_fp64_sources(const float *tile, const DfClass &k, int q, int real)
+__device__ __forceinline__ uint32_t df_fp64_sources(const float *tile, uint32_t direct, int q, int real)
 {
-    return (k.direct >> q) & 1u ? 0xffffffffu >> (kDfSub - real) : df_heavy<S>(tile, q);
+    return (direct >> q) & 1u ? 0xffffffffu >> (kDfSub - real) : df_heavy<S>(tile, q);
 }
+
+// The marked sources of a sub-block spread over a warp, the k-th of them on lane
+// k: this lane's source (the last one again past the end), and which of them is
+// the element `self` of the sub-block, this lane's target (-1: none).
+struct DfMarked {
+    int own, count, self;
+    __device__ __forceinline__ DfMarked(uint32_t marks, int64_t target)
+    {
+        count = __popc(marks);
+        self = target >= 0 && target < kDfSub && (marks >> (int)target & 1u)
+                   ? __popc(marks & ((1u << (int)target) - 1u)) : -1;
+        own = min((int)(threadIdx.x & 31u), count - 1);
+        if (marks & (marks + 1u)) own = (int)__fns(marks, 0, own + 1);   // (not the first `count` of them)
+    }
+};
+
+template <int S>
+__device__ __forceinline__ bool df_any_fp64(const float *tile, uint32_t direct, int n_sub)
+{
+    uint32_t any = direct;
+    for (int q = 0; q < n_sub; ++q) any |= df_heavy<S>(tile, q);
+    return any != 0;
+}
+
+// The softening of the FP64 pair terms, formed once per tile (the division alone is
+// some 20 FP64 instructions, most of a pair).
+struct DfSoftening {
+    double h2, hinv, hinv3, hinv5;
+    __device__ __forceinline__ explicit DfSoftening(double h)
+    {
+        h2 = h * h;
+        hinv = 1.0 / h;
+        hinv3 = hinv * hinv * hinv;
+        hinv5 = hinv3 * hinv * hinv;
+    }
+};
 
 __device__ __forceinline__ float df_diagonal2(const float *box)
 {
@@ -531,7 +567,7 @@ __device__ __forceinline__ DfClass df_classify(const float *tile, const DfHead &
     k.direct = 0;
     k.close = 0;
     k.rmin2 = 0x1p60f;
-    if (!(__all_sync(0xffffffffu, !live || at < kDfRange) && head.ok)) {
+    if (!__all_sync(0xffffffffu, !live || at < kDfRange)) {
         k.direct = (1u << n_sub) - 1u;
         return k;
     }
@@ -569,7 +605,7 @@ __device__ __forceinline__ DfClass df_classify(const float *tile, const DfHead &
 __device__ __forceinline__ double df_offset(const DfHead &head, const double c[3], const double x[3],
                                             DfTarget &tg)
 {
-    const double il = pow2d(head.ok ? -head.el : 0);
+    const double il = pow2d(-head.el);
     const double xs[3] = {__dmul_rn(__dsub_rn(x[0], c[0]), il), __dmul_rn(__dsub_rn(x[1], c[1]), il),
                           __dmul_rn(__dsub_rn(x[2], c[2]), il)};
     df_split(xs, tg);

@@ -141,7 +141,7 @@ __device__ __forceinline__ void df_pair_terms(double r2, double m, double h2, do
     } else {
         mg = mf * ri2;
     }
-    if (r2 < h2) {
+    if (__double_as_longlong(r2) < __double_as_longlong(h2)) {   // (r2 < h2, both not negative, off the FP64 unit)
         double F, Gp, P;
         spline_kernel<double>(sqrt(r2) * hinv, F, Gp, P);
         mf = m * F * hinv3;
@@ -181,31 +181,40 @@ __device__ __noinline__ void df_flush(const double *__restrict__ pos, const doub
 }
 
 // The marked sources of the sub-block at element `first` in FP64 from the
-// caller's arrays (every lane reads the same source): heavy sources, sub-blocks
-// inside the softening, tiles out of the two-part ranges.
+// caller's arrays: heavy sources, sub-blocks inside the softening, tiles out of the
+// two-part ranges.  Each lane loads one source, its velocity relative to the
+// tile's, and hands it round: the FP64 unit bounds this loop, and subtracting the
+// tile's velocity and comparing r^2 and h^2 in FP64 for every pair, and dividing
+// by h for every sub-block, cost a tenth (16384 elements, all pairs here: 21.3 ms,
+// now 19.0; eval_f64_kernel 19.2).
 template <bool POT>
 __device__ __forceinline__ void df_fp64_loop(const EvalArgs &a, const TileGeom &g, int64_t first,
-                                             uint32_t marks, const double xi[3], int64_t ti,
+                                             uint32_t marks, const double xi[3], int64_t ti, const DfSoftening &h,
                                              double acc[kNCPot])
 {
-    const double h2 = a.h * a.h, hinv = 1.0 / a.h;
-    const double hinv3 = hinv * hinv * hinv;
-    const double hinv5 = hinv3 * hinv * hinv;
-    const double cv[3] = {(double)g.cv[0], (double)g.cv[1], (double)g.cv[2]};
-#pragma unroll 2
-    for (; marks; marks &= marks - 1u) {
-        const int64_t j = first + __ffs(marks) - 1;
-        const double dx = a.pos[3 * j] - xi[0], dy = a.pos[3 * j + 1] - xi[1], dz = a.pos[3 * j + 2] - xi[2];
+    const DfMarked s(marks, ti - first);
+    const int64_t own = first + s.own;
+    double x[3], v[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        x[c] = a.pos[3 * own + c];
+        v[c] = a.vel[3 * own + c] - (double)g.cv[c];
+    }
+    const double m = a.mass[own];
+#pragma unroll 4
+    for (int k = 0; k < s.count; ++k) {
+        const double dx = __shfl_sync(0xffffffffu, x[0], k) - xi[0], dy = __shfl_sync(0xffffffffu, x[1], k) - xi[1],
+                     dz = __shfl_sync(0xffffffffu, x[2], k) - xi[2];
         double mf, mg, mp;
-        df_pair_terms<POT, false>(fma(dx, dx, fma(dy, dy, dz * dz)), a.mass[j], h2, hinv, hinv3, hinv5, mf, mg,
-                                  mp);
-        if (j == ti) {
+        df_pair_terms<POT, false>(fma(dx, dx, fma(dy, dy, dz * dz)), __shfl_sync(0xffffffffu, m, k), h.h2, h.hinv,
+                                  h.hinv3, h.hinv5, mf, mg, mp);
+        if (k == s.self) {
             mf = 0.0;
             mg = 0.0;
             mp = 0.0;
         }
-        accumulate_d<POT>(acc, dx, dy, dz, a.vel[3 * j] - cv[0], a.vel[3 * j + 1] - cv[1],
-                          a.vel[3 * j + 2] - cv[2], mf, mg, mp);
+        accumulate_d<POT>(acc, dx, dy, dz, __shfl_sync(0xffffffffu, v[0], k), __shfl_sync(0xffffffffu, v[1], k),
+                          __shfl_sync(0xffffffffu, v[2], k), mf, mg, mp);
     }
 }
 
@@ -256,9 +265,14 @@ __device__ __forceinline__ bool df_item(const EvalArgs &a, DfSmem<NT, S, POT> &s
             const float *tile = sm.stage[s];
             const DfHead head = *reinterpret_cast<const DfHead *>(tile);
             DfTarget tg;
-            const double il = df_offset(head, g.c, xi, tg);
-            const DfClass k = df_classify(tile, head, tg, live, a.h, il);
+            DfClass k;
             const int el = head.el, n_sub = (head.count + kDfSub - 1) / kDfSub;
+            if (head.ok) {
+                const double il = df_offset(head, g.c, xi, tg);
+                k = df_classify(tile, head, tg, live, a.h, il);
+            } else {
+                k.direct = (1u << n_sub) - 1u;
+            }
             const double vr[3] = {vi[0] - (double)g.cv[0], vi[1] - (double)g.cv[1],
                                   vi[2] - (double)g.cv[2]};
             double acc[kNCPot];
@@ -314,9 +328,12 @@ __device__ __forceinline__ bool df_item(const EvalArgs &a, DfSmem<NT, S, POT> &s
                 // beyond the softening m f = m g' r^2
                 acc[FSUM] = __dadd_rn(__dadd_rn(acc[TXX], acc[TYY]), acc[TZZ]);
             }
-            for (int q = 0; q < n_sub; ++q) {
-                const uint32_t marks = df_fp64_sources<S>(tile, k, q, min(kDfSub, head.count - kDfSub * q));
-                if (marks) df_fp64_loop<POT>(a, g, g.first + (int64_t)kDfSub * q, marks, xi, i, acc);
+            if (df_any_fp64<S>(tile, k.direct, n_sub)) {
+                const DfSoftening h(a.h);
+                for (int q = 0; q < n_sub; ++q) {
+                    const uint32_t marks = df_fp64_sources<S>(tile, k.direct, q, min(kDfSub, head.count - kDfSub * q));
+                    if (marks) df_fp64_loop<POT>(a, g, g.first + (int64_t)kDfSub * q, marks, xi, i, h, acc);
+                }
             }
             target_velocity_d(acc, vr);
 #pragma unroll
