@@ -303,7 +303,7 @@ __device__ __forceinline__ bool bwd_df_item(const BwdArgs &a, BwdDfSmem<NT, S> &
             const int el = head.el, n_sub = (head.count + kDfSub - 1) / kDfSub;
             if (head.ok) {
                 const double il = df_offset(head, g.c, xk, tg);
-                k = df_classify(tile, head, tg, live, h, il);
+                k = df_classify<S, false>(tile, head, tg, live, h, il);
             } else {
                 k.direct = (1u << n_sub) - 1u;
             }

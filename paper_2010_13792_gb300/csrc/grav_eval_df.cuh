@@ -269,7 +269,7 @@ __device__ __forceinline__ bool df_item(const EvalArgs &a, DfSmem<NT, S, POT> &s
             const int el = head.el, n_sub = (head.count + kDfSub - 1) / kDfSub;
             if (head.ok) {
                 const double il = df_offset(head, g.c, xi, tg);
-                k = df_classify(tile, head, tg, live, a.h, il);
+                k = df_classify<S, true>(tile, head, tg, live, a.h, il);
             } else {
                 k.direct = (1u << n_sub) - 1u;
             }
