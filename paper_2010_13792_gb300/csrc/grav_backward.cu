@@ -939,7 +939,7 @@ __global__ void __launch_bounds__(256) backward_pot_only_kernel(const BwdArgs a)
 // Fixed tile shapes of the adjoint.
 constexpr int kBwdNTf = 768, kBwdKTf = 1, kBwdSf = 256, kBwdMinBf = 1, kBwdUf = 4;
 constexpr size_t kBwdSmemf = sizeof(BwdPairSmem<kBwdSf>);
-// FP64: 256-source tiles, 128 below 2^25 pairs (as the forward: kFinePairs)
+// FP64: 256-source tiles, 128 below 2^25 pairs (the forward's line, kFinePairs, is 2^26)
 constexpr int kBwdNTd = 128, kBwdSd = 256, kBwdSfine = 128, kBwdMinBd = 4;
 constexpr int64_t kBwdFinePairs = 1LL << 25;
 constexpr size_t kBwdSmemd = sizeof(BwdDfSmem<kBwdNTd, kBwdSd>);
@@ -953,6 +953,19 @@ struct BwdLayout {
 bool bwd_fine(const grav_params *p, int64_t n)
 {
     return p->precision == GRAV_F64 && p->max_split != 1 && n * n < kBwdFinePairs;
+}
+
+// The smallest (up to half an item, target block x tile, an SM: 1024 elements)
+// keep FP64 pair terms: each SM runs one CTA or none, so a call takes as long as
+// its slowest item, and a tile that takes both routes, two parts and FP64 sources,
+// takes the sum of both (a_bar = -x, FP64 pairs / both / FP64 throughout: 500 elements 207 /
+// 251 / 191 us, 1000 223 / 242 / 193; like a_bar 1536 344 / 212 / 298).
+bool bwd_few(const grav_params *p, int64_t n)
+{
+    int sms = 0;
+    if (device_sm_count(&sms) != GRAV_OK) return false;
+    const int64_t items = ((n + kBwdNTd - 1) / kBwdNTd) * ((n + kBwdSfine - 1) / kBwdSfine);
+    return bwd_fine(p, n) && 2 * items <= sms;
 }
 
 int bwd_layout(const grav_params *p, int64_t n, BwdLayout *L)
@@ -1159,7 +1172,8 @@ extern "C" int grav_eval_backward(const grav_params *p, int64_t n, const double 
             const_cast<float *>(a.src_lo));
     else if (fine)
         pack_tiles_kernel<kBwdSfine, false, false, false, true><<<(unsigned)L.n_tiles, kBwdSfine, 0, st>>>(
-            n, pos, a_bar, nullptr, const_cast<TileGeom *>(a.geo), const_cast<void *>(a.src), flags_dev);
+            n, pos, a_bar, nullptr, const_cast<TileGeom *>(a.geo), const_cast<void *>(a.src), flags_dev, nullptr,
+            bwd_few(p, n));
     else
         pack_tiles_kernel<kBwdSd, false, false, false, true><<<(unsigned)L.n_tiles, kBwdSd, 0, st>>>(
             n, pos, a_bar, nullptr, const_cast<TileGeom *>(a.geo), const_cast<void *>(a.src), flags_dev);

@@ -114,11 +114,13 @@ __device__ __forceinline__ float df_heavy_line(float net, float gross, float squ
 // Packs one tile (one CTA of S threads, thread j its source): `x` the FP64
 // offset from the tile centre, `v` the velocity relative to the tile's
 // velocity centre (ADJ: the adjoint's a_bar), m the mass; `half` the tile's half
-// extents; `alone`: the system has no other tile.  Padding sources (!ok) copy the
+// extents; `alone`: the system has no other tile; all_fp64: the caller wants every
+// tile summed in FP64.  Padding sources (!ok) copy the
 // place of their sub-block's first source with zero mass.  A warp is a sub-block.
 template <int S, bool ADJ>
-__device__ __forceinline__ void df_pack(void *tile, int j, bool ok, int count, bool alone, const double x[3],
-                                        const double v[3], double m, const double half[3], double cmax)
+__device__ __forceinline__ void df_pack(void *tile, int j, bool ok, int count, bool alone, bool all_fp64,
+                                        const double x[3], const double v[3], double m, const double half[3],
+                                        double cmax)
 {
     constexpr int W = S / 32;
     __shared__ uint32_t wtop[2][W], wlight[3][W];
@@ -165,7 +167,7 @@ __device__ __forceinline__ void df_pack(void *tile, int j, bool ok, int count, b
     if (hx == 0 && hc == 0) el = 0;
     const int em = top[0] == 0 ? 0 : exponent_above(top[0]), ev = top[1] == 0 ? 0 : exponent_above(top[1]);
     bool good = hx < 0x7ff00000u && top[0] < 0x7ff00000u && top[1] < 0x7ff00000u && abs(el) <= 150 &&
-                abs(em) <= 150 && abs(ev) <= 150 && !(alone && count <= kDfFewest);
+                abs(em) <= 150 && abs(ev) <= 150 && !(alone && count <= kDfFewest) && !all_fp64;
     el = max(-150, min(150, el));
     h.el = (int16_t)el;
     // heavy sources

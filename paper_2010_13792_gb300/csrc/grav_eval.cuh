@@ -377,7 +377,7 @@ __device__ __forceinline__ void pack_tile(int t, int64_t first, int64_t end,
                                           const double *__restrict__ mass,
                                           TileGeom *__restrict__ geo, void *__restrict__ src,
                                           int32_t *flags, float *__restrict__ src_lo = nullptr,
-                                          bool alone = false)
+                                          bool alone = false, bool all_fp64 = false)
 {
     constexpr int NV = VOFF ? 6 : 3;      // boxes of the positions and, with VOFF, the velocities
     __shared__ double mm[2 * NV];
@@ -475,7 +475,8 @@ __device__ __forceinline__ void pack_tile(int t, int64_t first, int64_t end,
             half[c] = fmax(__dsub_ru(mm[2 * c + 1], cc[c]), __dsub_ru(cc[c], mm[2 * c]));
         const double cmax = fmax(fabs(cc[0]), fmax(fabs(cc[1]), fabs(cc[2])));
         df_pack<S, !VOFF>(static_cast<char *>(src) + (int64_t)t * df_stride<S>(), j, ok,
-                          (int)(end - first < S ? end - first : S), alone, off, vo, m, half, cmax);
+                          (int)(end - first < S ? end - first : S), alone, all_fp64, off, vo, m, half,
+                          cmax);
     } else {
         D4 *tile = static_cast<D4 *>(src) + (int64_t)t * 2 * S;
         D4 pm, pv;
@@ -508,12 +509,12 @@ template <int S, bool MIXED, bool VOFF, bool PAIR = false, bool DF = false>
 __global__ void __launch_bounds__(S)
 pack_tiles_kernel(int64_t n_src, const double *__restrict__ pos, const double *__restrict__ vel,
                   const double *__restrict__ mass, TileGeom *__restrict__ geo, void *__restrict__ src,
-                  int32_t *flags, float *__restrict__ src_lo = nullptr)
+                  int32_t *flags, float *__restrict__ src_lo = nullptr, bool all_fp64 = false)
 {
     const int64_t first = (int64_t)blockIdx.x * S;
     const int64_t end = first + S < n_src ? first + S : n_src;
     pack_tile<S, MIXED, VOFF, PAIR, DF>(blockIdx.x, first, end, pos, vel, mass, geo, src, flags,
-                                        src_lo, n_src <= S);
+                                        src_lo, n_src <= S, all_fp64);
 }
 
 // ---------------------------------------------------------------------------
