@@ -180,12 +180,15 @@ constexpr int64_t kFinePairs = 1LL << 26;
 int tile_kind(const grav_params *p, const EvalConfig *c, int mode, int64_t n_src, int64_t n_idx_max)
 {
     if (c->precision != GRAV_F64 || mode != kModeOpen || p->max_split == 1) return kNominal;
-    // The smallest keep FP64 pair terms: a sub-block of 32 of a few thousand
-    // elements is so long that most pairs of a concentrated system count as
-    // close and are summed in FP64 anyway.  Up to two items (target block x
-    // tile) an SM, and from three, the two-part kernel's residency, to four, where
-    // its second round is nearly empty (Plummer, FP64 / two-part: 500 elements 234 /
-    // 288 us, 2139 409 / 460, 2500 591 / 485, 2900 753 / 833, 3500 1172 / 895).
+    // The smallest keep FP64 pair terms: most pairs of a few thousand elements of
+    // a concentrated system are close and summed in FP64 anyway, and a call of few
+    // items is as long as its slowest.  Up to two items (target block x tile) an SM, and
+    // from three, the two-part kernel's residency in the default configuration, to
+    // four, where its second round is nearly empty (Plummer, FP64 / two-part: 500
+    // elements 234 / 288 us, 2139 409 / 460, 2500 591 / 485, 2900 753 / 833, 3500 1172 / 895).  Configurations 1
+    // and 2 (six CTAs and one an SM) keep the default's line: with their own residency
+    // configuration 1 took 783 instead of 1032 us at 2900 elements of a Plummer sphere, but 784
+    // instead of 540 of a uniform one.
     int sms = 0;
     if (device_sm_count(&sms) != GRAV_OK) sms = 152;
     const int64_t BT = (int64_t)c->threads * c->kt;
