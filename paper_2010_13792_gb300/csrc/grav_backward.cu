@@ -165,7 +165,7 @@ __device__ __forceinline__ void bwd_pair_fp64(const double d[3], const double ab
     const double ri2 = ri * ri;
     double f = ri * ri2;
     double gp = f * ri2;
-    if (__double_as_longlong(r2) < __double_as_longlong(h2)) {   // (as df_pair_terms)
+    if (less_bits(r2, h2)) {
         double F, Gp, P;
         spline_kernel<double>(sqrt(r2) * hinv, F, Gp, P);
         f = F * hinv3;

@@ -94,6 +94,14 @@ __device__ __forceinline__ void two_sum_ordered(double &hi, double &lo, double x
     hi = t;
 }
 
+// a < b on the integer side (the FP64 unit runs at 1/64 of its rate) for a and b
+// that are not negative; false where a is NaN.  Unsigned: the NaN of an FP64
+// operation may carry the sign.
+__device__ __forceinline__ bool less_bits(double a, double b)
+{
+    return (unsigned long long)__double_as_longlong(a) < (unsigned long long)__double_as_longlong(b);
+}
+
 __device__ __forceinline__ uint32_t smem_addr(const void *p)
 {
     return static_cast<uint32_t>(__cvta_generic_to_shared(p));

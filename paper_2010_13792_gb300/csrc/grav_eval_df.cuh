@@ -141,7 +141,7 @@ __device__ __forceinline__ void df_pair_terms(double r2, double m, double h2, do
     } else {
         mg = mf * ri2;
     }
-    if (__double_as_longlong(r2) < __double_as_longlong(h2)) {   // (r2 < h2, both not negative, off the FP64 unit)
+    if (less_bits(r2, h2)) {
         double F, Gp, P;
         spline_kernel<double>(sqrt(r2) * hinv, F, Gp, P);
         mf = m * F * hinv3;

@@ -365,9 +365,10 @@ __global__ void __launch_bounds__(kSoftNT) soft_solve_kernel(SoftArgs a)
             // r / h rounds to 1, where every term is zero)
             uint8_t in[kSoftList];
             int n_in = 0;
-            const long long hb = __double_as_longlong(h);        // (non-negative: ordered as integers)
+            // (an element without a place, a NaN, lists every source and the last
+            // tile's padding: none of them is in reach, and padding has no mass to read)
             for (int k = 0; k < cnt; ++k)
-                if (__double_as_longlong(nr[k]) < hb) in[n_in++] = (uint8_t)k;
+                if (less_bits(nr[k], h) && nj[k] < a.n) in[n_in++] = (uint8_t)k;
             for (int q = 0; q < n_in; ++q) {
                 const int k = in[q];
                 const int32_t j = nj[k];
