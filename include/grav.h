@@ -396,7 +396,9 @@ typedef struct grav_soft_params {
  *   out): device, out, each nullable
  * A mass or guess that is not positive and finite sets GRAV_FLAG_NONFINITE
  * and leaves that element's outputs unwritten.
- * workspace: >= grav_soft_workspace_bytes(n) bytes, 256-byte aligned.
+ * workspace: >= grav_soft_workspace_bytes(n) bytes, 256-byte aligned.  The kernel
+ * also keeps neighbour lists of 1.9 KB a thread in local memory, for which the
+ * driver sets some 0.6 GB (152 SMs) of the device aside at its first launch.
  */
 GRAV_API int64_t grav_soft_workspace_bytes(int64_t n);
 GRAV_API int grav_soft_solve(const grav_soft_params *sp, int64_t n, const double *pos,

@@ -27,10 +27,15 @@
 // warp run the FP64 terms side by side: FP64 bounds this kernel, and with the
 // terms inside the scan a warp ran them once for every source inside any of
 // its 32 supports, 12 lanes active (40961 elements, n_ngb = 32, guesses off by
-// up to 20%: 8.1 ms, with the lists 3.0 ms).  An element with more than
-// kSoftList sources in reach sums them in the scans.  Every order of summation
-// is that of the sources.  Newton steps are limited to a factor of 2 in h.
-// Every loop is bounded by max_iter passes.
+// up to 20%: 8.1 ms, with the lists 3.0 ms).  Where a list would be full the
+// element is summed in the scan; every scan counts the sources in reach, which
+// tells the next pass, so a pass takes one scan unless a list overflows against
+// the estimate (a Plummer sphere of 40961, guesses off by up to 20%, sums in the
+// scans alone / two lists tried in every pass / this: n_ngb = 32 8.5 / 7.8 / 6.0 ms, 64 17.9 / 36.5 /
+// 18.5, 128 98 / 135 / 100, 300 315 / 372 / 319; guesses twice too large, n_ngb = 32, 230 / 271 / 233).
+// Every order of summation is that of the sources.  Newton steps are limited to a
+// factor of 2 in h.
+// Every loop is bounded: max_iter passes of at most three scans.
 #include <cmath>
 
 #include "grav_common.cuh"
@@ -194,6 +199,14 @@ __device__ __forceinline__ bool box_near(const float blo[3], const float bhi[3],
 
 constexpr int kSoftList = 144;      // listed sources per element (local memory)
 constexpr double kSoftReach = 1.2;  // list radius over the support it is made for
+constexpr float kSoftSure = 0.84f;  // (0.84^3 = 0.6 of kSoftList expected: room for a gradient of density)
+
+// The radius at which the list would be full, from `count` sources within r of
+// an element (uniform density; an estimate, the scan counts again).
+__device__ __forceinline__ float soft_fill(double r, float count)
+{
+    return __double2float_rn(r) * cbrtf((float)kSoftList / fmaxf(count, 1.0f));
+}
 
 __global__ void __launch_bounds__(kSoftNT) soft_solve_kernel(SoftArgs a)
 {
@@ -226,18 +239,38 @@ __global__ void __launch_bounds__(kSoftNT) soft_solve_kernel(SoftArgs a)
     double nr[kSoftList];
     int cnt = 0;
     double reach = 0.0;
+    // radii from which a list is not tried: where it would be full by the last
+    // count (first by n_ngb, as if the guess were right), and what overflowed
+    float fill = soft_fill(h, (float)a.n_ngb), over = inf;
+    bool fresh = false;                // the distances of the list are still to be formed
 
     for (int pass = 0; pass < a.max_iter; ++pass) {
         if (!__syncthreads_or(!done)) break;       // every element of the CTA is done
         double rho = 0.0, rho_h = 0.0, psi_h = 0.0;
         const double hinv = 1.0 / h, h2 = h * h;
-        // ---- scans: lists for the supports that outgrew theirs; one that
-        // overflows is made for the support alone in a second scan, and when
-        // that overflows too a third scan sums the element directly
-        bool want = !done && h > reach, direct = false;
-        double factor = kSoftReach;
-        while (__syncthreads_or(want)) {
-            const double rad = factor * h;
+        // ---- scans for the supports that outgrew their list.  A list of the
+        // support and a fifth, or of the support alone, where the last count
+        // leaves room to spare; otherwise the element is summed in the scan
+        // (direct), which records what is inside the support on the way if that
+        // may fit.  A list that overflows against the estimate takes the next
+        // choice in another scan.  Elements summed in one scan share its FP64
+        // terms, so where a sixteenth of the CTA's are, all are.
+        bool want = !done && h > reach, direct = false, record = false;
+        double rad = h;
+        auto choose = [&] {
+            const float most = fminf(fill, 0.95f * over), hr = __double2float_ru(h);
+            direct = hr > kSoftSure * most;
+            rad = (float)kSoftReach * hr <= kSoftSure * most ? kSoftReach * h : h;
+            record = hr <= most;
+        };
+        if (want) choose();
+        for (;;) {
+            const int wanting = __syncthreads_count(want), summing = __syncthreads_count(want && direct);
+            if (wanting == 0) break;
+            if (want && !direct && 16 * summing >= wanting) {
+                direct = record = true;
+                rad = h;
+            }
             float l[3], u[3], hm = want ? __double2float_ru(rad) : 0.0f;
             for (int c = 0; c < 3; ++c) {
                 l[c] = want ? __double2float_rd(xi[c]) : inf;
@@ -278,7 +311,7 @@ __global__ void __launch_bounds__(kSoftNT) soft_solve_kernel(SoftArgs a)
             const float B_lo[3] = {blo[0], blo[1], blo[2]}, B_hi[3] = {bhi[0], bhi[1], bhi[2]};
             const float H = bh;
             const bool any_direct = __syncthreads_or(want && direct) != 0;
-            if (want && !direct) cnt = 0;
+            if (want) cnt = 0;
             const float hf = __double2float_ru(rad);
             const float hlim2 = __fmul_ru(hf, hf);
             for (int64_t t0 = 0; t0 < a.n_tiles; t0 += kSoftNT) {
@@ -317,25 +350,33 @@ __global__ void __launch_bounds__(kSoftNT) soft_solve_kernel(SoftArgs a)
                             const float err = __fmul_ru(__fadd_ru(tb.ext, tmax), 0x1p-21f);
                             const float hl = __fadd_ru(hf, __fmul_ru(err, 1.8f));
                             const float lim = __fmul_ru(__fmul_ru(hl, hl), 1.0f + 0x1p-20f);
+                            if (!direct) {
 #pragma unroll 4
-                            for (int j = 0; j < kSoftS; ++j) {
-                                const float4 q = sx32[j];
-                                const float ex = q.x - tq[0], ey = q.y - tq[1], ez = q.z - tq[2];
-                                if (fmaf(ex, ex, fmaf(ey, ey, ez * ez)) >= lim) continue;
-                                if (!direct) {
+                                for (int j = 0; j < kSoftS; ++j) {
+                                    const float4 q = sx32[j];
+                                    const float ex = q.x - tq[0], ey = q.y - tq[1], ez = q.z - tq[2];
+                                    if (fmaf(ex, ex, fmaf(ey, ey, ez * ez)) >= lim) continue;
                                     if (cnt < kSoftList) nj[cnt] = (int32_t)(t * kSoftS + j);
                                     ++cnt;
-                                    continue;
                                 }
-                                const double4 s = sx[j];
-                                const double dx = s.x - xi[0], dy = s.y - xi[1], dz = s.z - xi[2];
-                                const double r2 = fma(dx, dx, fma(dy, dy, dz * dz));
-                                if (r2 < h2) {
-                                    double w, wh, ph;
-                                    density_terms(sqrt(r2) * hinv, hinv, w, wh, ph);
-                                    rho = fma(s.w, w, rho);
-                                    rho_h = fma(s.w, wh, rho_h);
-                                    if (t * kSoftS + j != i) psi_h = fma(s.w, ph, psi_h);
+                            } else {
+#pragma unroll 4
+                                for (int j = 0; j < kSoftS; ++j) {
+                                    const float4 q = sx32[j];
+                                    const float ex = q.x - tq[0], ey = q.y - tq[1], ez = q.z - tq[2];
+                                    if (fmaf(ex, ex, fmaf(ey, ey, ez * ez)) >= lim) continue;
+                                    if (record && cnt < kSoftList) nj[cnt] = (int32_t)(t * kSoftS + j);
+                                    ++cnt;
+                                    const double4 s = sx[j];
+                                    const double dx = s.x - xi[0], dy = s.y - xi[1], dz = s.z - xi[2];
+                                    const double r2 = fma(dx, dx, fma(dy, dy, dz * dz));
+                                    if (r2 < h2) {
+                                        double w, wh, ph;
+                                        density_terms(sqrt(r2) * hinv, hinv, w, wh, ph);
+                                        rho = fma(s.w, w, rho);
+                                        rho_h = fma(s.w, wh, rho_h);
+                                        if (t * kSoftS + j != i) psi_h = fma(s.w, ph, psi_h);
+                                    }
                                 }
                             }
                         }
@@ -344,23 +385,31 @@ __global__ void __launch_bounds__(kSoftNT) soft_solve_kernel(SoftArgs a)
                 }
             }
             if (want) {
-                if (!direct && cnt > kSoftList) {
-                    direct = factor == 1.0;
-                    factor = 1.0;
-                } else {
-                    want = false;
-                    reach = direct ? 0.0 : rad;
-                    for (int k = 0; k < (direct ? 0 : cnt); ++k) {
-                        const double4 s = a.src[nj[k]];
-                        const double dx = s.x - xi[0], dy = s.y - xi[1], dz = s.z - xi[2];
-                        nr[k] = sqrt(fma(dx, dx, fma(dy, dy, dz * dz)));
-                    }
+                fill = soft_fill(rad, (float)cnt);
+                const bool fits = cnt <= kSoftList;
+                if (!fits && (!direct || record)) over = fminf(over, __double2float_rn(rad));
+                want = !direct && !fits;
+                reach = fits && (!direct || record) ? rad : 0.0;
+                fresh = true;
+                if (want) {
+                    // the support alone after a support and a fifth, else direct: at
+                    // most three scans, whatever the radii round to in FP32
+                    const bool last = !(rad > h);
+                    choose();
+                    direct = direct || last || rad > h;
+                    rad = h;
                 }
             }
         }
 
         // ---- sums over the listed sources inside the support ----
         if (!done && !direct) {
+            for (int k = 0; fresh && k < cnt; ++k) {
+                const double4 s = a.src[nj[k]];
+                const double dx = s.x - xi[0], dy = s.y - xi[1], dz = s.z - xi[2];
+                nr[k] = sqrt(fma(dx, dx, fma(dy, dy, dz * dz)));
+            }
+            fresh = false;
             // (r < h where the scan asks r^2 < h^2: the two differ at most where
             // r / h rounds to 1, where every term is zero)
             uint8_t in[kSoftList];
