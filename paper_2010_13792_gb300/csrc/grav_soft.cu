@@ -199,7 +199,11 @@ __device__ __forceinline__ bool box_near(const float blo[3], const float bhi[3],
 
 constexpr int kSoftList = 144;      // listed sources per element (local memory)
 constexpr double kSoftReach = 1.2;  // list radius over the support it is made for
-constexpr float kSoftSure = 0.84f;  // (0.84^3 = 0.6 of kSoftList expected: room for a gradient of density)
+// A list is tried up to this share of the radius where it would be full: 0.75 of
+// kSoftList expected, room for a gradient of density (Plummer sphere of 40961 /
+// uniform cloud of 200003, n_ngb = 64, right / too small guesses: 0.84 2.4 / 15.4 ms, 0.91 2.4 /
+// 10.5, 0.95 3.6 / 8.6).
+constexpr float kSoftSure = 0.91f;
 
 // The radius at which the list would be full, from `count` sources within r of
 // an element (uniform density; an estimate, the scan counts again).
