@@ -70,7 +70,8 @@ extern "C" {
                          terms that cancel and systems of up to 128 elements stay in FP64
                          (csrc/grav_df.cuh).  An output is within about 2e-15 of the sum of
                          its terms' magnitudes (the jerk's taken with the largest relative
-                         velocity), as with FP64 pair terms throughout. */
+                         velocity); its error is 1.5 to 2 times that of FP64 pair terms in
+                         the median, up to ten times at single targets whose sums cancel. */
 #define GRAV_MIXED 1  /* FP64 positions offset to FP32 per source tile, FP32 pair
                          arithmetic, compensated FP32 tile sums, FP64 final sums */
 
@@ -91,7 +92,8 @@ typedef struct grav_params {
 typedef struct grav_tile_info {
     int32_t threads;          /* threads per CTA */
     int32_t targets_per_thread;
-    int32_t sources_per_tile; /* S: sources staged per shared-memory tile */
+    int32_t sources_per_tile; /* S: sources staged per shared-memory tile (GRAV_F64 with open
+                                 boundaries and many pairs: 2 S) */
     int32_t targets_per_block;/* threads * targets_per_thread */
     int32_t unroll;           /* unroll depth of the Newtonian pair loop (mixed), 0 if fixed */
     int32_t shared_accumulators; /* 1: compensated sums kept in shared memory */

@@ -3,7 +3,8 @@
 // GB300 runs FP64 at 1/64 of its FP32 rate (2 FMA per clock and SM), and the
 // FP64 force kernel needs 39 FP64 instructions a pair: 2500 FP32 lane slots.
 // The same pair carried as unevaluated sums of two FP32 numbers (about 48 bits)
-// takes some 190 FP32 operations, two sources to a packed FP32x2 instruction.
+// takes some 320 FP32 operations, two sources to a packed FP32x2 instruction
+// (ncu: 203 warp instructions a pair with everything around them).
 //
 // Pieces:
 //   * Tiles hold the sources' offsets from the tile centre in units of a power

@@ -4,9 +4,10 @@
 // barrier between tiles); the running FP64 sums (hi, lo) of each target in
 // shared memory.
 //
-// What bounds it: the FP32 pipe (about 270 lane operations a pair); the FP64
-// unit is busy with the per-tile conversions and carries, about 160 FP64
-// instructions per warp and tile, beside the other warps' FP32 work.
+// What bounds it: issue and the FP32 pipe's latency (about 320 lane operations a
+// pair in dependent chains, 12 warps an SM by registers: issue slots 43% busy, 1.81
+// instructions a clock); the FP64 unit, 23% busy, has the per-tile conversions and
+// carries, about 160 FP64 instructions per warp and tile, and the listed pairs.
 #pragma once
 
 #include "grav_df.cuh"
