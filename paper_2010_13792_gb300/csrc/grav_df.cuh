@@ -487,13 +487,14 @@ constexpr float kDfLeast2 = 0x1p-44f;
 // costs more than summing the sub-block in FP64.  So the forward counts them first
 // (FP32, 2% of a sub-block's two-part sums), and above this share the sub-block goes
 // to FP64.  Plummer spheres in random order, FP64 pairs / listed / by this rule:
-// 16384 elements 19.7 / 25.7 / 19.1 ms, 65536 312 / 407 / 302 ms; in Morton order 65536
-// 54.8 -> 54.6 ms.  Shares from 0.2 to 0.5 do alike, from 0.65 a uniform sphere loses it.
+// 16384 elements 19.7 / 25.7 / 20.6 ms, 65536 312 / 407 / 326 ms; in Morton order 65536
+// 54.8 ms either way.  Shares from 0.2 to 0.5 do alike, from 0.65 a uniform sphere loses it.
 // The adjoint lists: 12289 7.64 ms against 7.74 in FP64 tiles.
 constexpr float kDfLoose = 0.25f;
 
 struct DfClass {
     uint32_t direct;   // sub-blocks summed in FP64 (softening wider than half their diagonal, kDfLeast2)
+    uint32_t loose;    // of these, those with too many pairs to list
     uint32_t close;    // sub-blocks with listed pairs
     float rmin2;       // least r^2 of the pairs left to this lane's target
     float floor2;      // least listing radius (squared)
@@ -598,6 +599,7 @@ __device__ __forceinline__ DfClass df_classify(const float *tile, const DfHead &
     const int n_sub = (head.count + kDfSub - 1) / kDfSub;
     k.floor2 = fmaxf(hl * hl * (1.0f + 0x1p-18f), ext2 * 0x1p-8f);
     k.direct = 0;
+    k.loose = 0;
     k.close = 0;
     k.rmin2 = 0x1p60f;
     if (!__all_sync(0xffffffffu, !live || at < kDfRange)) {
@@ -631,6 +633,7 @@ __device__ __forceinline__ DfClass df_classify(const float *tile, const DfHead &
                 const int near = __reduce_add_sync(0xffffffffu, live ? df_count_close<S>(tile, q, real, tg, thr2) : 0);
                 if ((float)near > kDfLoose * (float)(real * __popc(__ballot_sync(0xffffffffu, live)))) {
                     k.direct |= 1u << q;
+                    k.loose |= 1u << q;
                     continue;
                 }
             }

@@ -2,8 +2,9 @@
 half: a sub-block of 32 sources then spans the system, and most of its pairs count
 as close.  The sums hold to 2e-13 of the sum of their terms' magnitudes
 (test_gpu_df), and the order costs no more than summing every pair in FP64 does:
-the same elements with masses out of the two-part range.  (They agree to a percent;
-listing the pairs one by one took 1.21 times as long.  The line is half way.)"""
+the same elements with masses out of the two-part range.  (They agree to a percent
+or, with the target's velocity in every pair, to eight; listing the pairs one by one
+took 1.21 times as long.)"""
 import numpy as np
 import pytest
 import torch
