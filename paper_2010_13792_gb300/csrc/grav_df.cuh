@@ -101,7 +101,11 @@ __device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b
 // 1.1e-15 / 1.4e-16; one mass of 1 among 299 of 1e-12, at it, 3.8e-16 / 3.1e-9 /
 // 6.8e-16; the adjoint's largest error for a random a_bar 3e-15 / 6e-14 / 3e-15.
 // 16384 elements: 4.4 ms, with that mass function 5.1 ms.
-constexpr int kDfAverage = 64;
+// For an a_bar K = 16 (2e-15 of the tile's sum): in the middle of a smooth field it
+// points to all sides, and |sum| is a third of the sum of its norms; such a tile is one
+// of many.  A smooth loss, forward and adjoint, K = 64 / 16: sphere of 1771 908 / 841 us, cloud of
+// 3000 1434 / 1288 us, with the same errors; random signs still go to FP64.
+constexpr int kDfAverage = 64, kDfAverageAdj = 16;
 constexpr int kDfFewest = 128;
 
 // (the larger side of the rule: heavier than this)
@@ -200,7 +204,7 @@ __device__ __forceinline__ void df_pack(void *tile, int j, bool ok, int count, b
 #pragma unroll
         for (int k = 0; k < W; ++k) sum[q] += wsum[q][k];
     }
-    const float K = fminf((float)kDfAverage, 0.5f * (float)count);
+    const float K = fminf((float)(ADJ ? kDfAverageAdj : kDfAverage), 0.5f * (float)count);
     const float net_v = ADJ ? sqrtf(fmaf(sum[3], sum[3], fmaf(sum[4], sum[4], sum[5] * sum[5]))) : sum[6];
     bool heavy = un > df_heavy_line(net_v, sum[6], sum[7], K, good);
     if (!ADJ) heavy = fabsf(w) > df_heavy_line(fabsf(sum[0]), sum[1], sum[2], K, good) || heavy;
