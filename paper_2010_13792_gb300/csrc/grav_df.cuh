@@ -492,9 +492,11 @@ constexpr float kDfLeast2 = 0x1p-44f;
 // (FP32, 2% of a sub-block's two-part sums), and above this share the sub-block goes
 // to FP64.  Plummer spheres in random order, FP64 pairs / listed / by this rule:
 // 16384 elements 19.7 / 25.7 / 20.6 ms, 65536 312 / 407 / 326 ms; in Morton order 65536
-// 54.8 ms either way.  Shares from 0.2 to 0.5 do alike, from 0.65 a uniform sphere loses it.
+// 54.8 ms either way.  Shares from 0.2 to 0.5 do alike in random order, from 0.65 a
+// uniform sphere loses it; in Morton order 0.35 lists more of the nearest sub-blocks
+// than 0.25 (cloud of 6794 1.48 -> 1.41 ms).
 // The adjoint lists: 12289 7.64 ms against 7.74 in FP64 tiles.
-constexpr float kDfLoose = 0.25f;
+constexpr float kDfLoose = 0.35f;
 
 struct DfClass {
     uint32_t direct;   // sub-blocks summed in FP64 (softening wider than half their diagonal, kDfLeast2)
