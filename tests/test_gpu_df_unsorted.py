@@ -2,8 +2,9 @@
 half: a sub-block of 32 sources then spans the system, and most of its pairs count
 as close.  The sums hold to 2e-13 of the sum of their terms' magnitudes
 (test_gpu_df), and the order costs no more than summing every pair in FP64 does:
-the same elements with masses out of the two-part range.  (With the target's velocity in every pair the order
-costs 1.09 times as much; listing the pairs one by one 1.17 to 1.28 times.)"""
+the same elements with masses out of the two-part range.  (With the target's
+velocity in every pair it costs 1.09 times as much, with every pair listed 1.17 to
+1.28 times.)"""
 import numpy as np
 import pytest
 import torch
